@@ -15,6 +15,7 @@
 
 #include "d3q19.cuh"
 #include "lbm_internal.h"
+#include "reduce.cuh"
 
 namespace lbm {
 
@@ -777,47 +778,141 @@ template <typename T> __device__ __forceinline__ T tforce_of(const SweepArgs& a,
 template <> __device__ __forceinline__ double tforce_of<double>(const SweepArgs& a, int i) { return a.tforce[i]; }
 template <> __device__ __forceinline__ float tforce_of<float>(const SweepArgs& a, int i) { return a.tforcef[i]; }
 
-// Deterministic block sum of four doubles; thread 0 of the block gets the totals.
-__device__ __forceinline__ void block_sum4(double (&v)[4], double* out) {
-  __shared__ double red[SWEEP_THREADS / 32][4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) red[warp][j] = v[j];
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t[4] = {0, 0, 0, 0};
-    for (int w = 0; w < SWEEP_THREADS / 32; ++w)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) t[j] += red[w][j];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) out[j] = t[j];
-  }
+// What a node contributes to the residual reductions: the density deviation, the
+// velocity and the snapshot's velocity.
+template <typename T>
+struct NodeTerms {
+  T drho, u[3], p[3];
+};
+
+// Reads the snapshot; block_terms replaces it by the current velocity.
+template <typename T>
+__device__ __forceinline__ NodeTerms<T> residual_terms(const Moments<T>& m, const T* snap, uint32_t N, uint32_t cell) {
+  return {m.drho, {m.ux, m.uy, m.uz}, {snap[cell], snap[N + cell], snap[2ull * N + cell]}};
+}
+// Called behind a block barrier that follows the first use of the snapshot's values: a
+// store issued while a load of the same address is in flight stalls the memory pipe (a
+// residual step on 512^3 FP32 took 14.8 ms with the stores right behind the loads).
+template <typename T>
+__device__ __forceinline__ void store_snapshot(const NodeTerms<T>& t, T* snap, uint32_t N, uint32_t cell) {
+  snap[cell] = t.u[0];
+  snap[N + cell] = t.u[1];
+  snap[2ull * N + cell] = t.u[2];
 }
 
-// Per-node contributions to the residual reductions: mass, |u - u_snap|^2, |u|^2 and
-// a bad-node flag; replaces the snapshot by the current velocity.
+// The four sums in double: sum of drho, |u - p|^2, |u|^2 and a bad-node flag.
 template <typename T>
-__device__ __forceinline__ void residual_terms(const Moments<T>& m, double rho0, T* snap, uint32_t N,
-                                               uint32_t cell, double (&v)[4]) {
-  const double rho = rho0 + double(m.drho);
-  const double u[3] = {double(m.ux), double(m.uy), double(m.uz)};
-  const double p[3] = {double(snap[cell]), double(snap[N + cell]), double(snap[2ull * N + cell])};
-  snap[cell] = m.ux;
-  snap[N + cell] = m.uy;
-  snap[2ull * N + cell] = m.uz;
-  v[0] = rho;
-  const double d0 = op_sub(u[0], p[0]), d1 = op_sub(u[1], p[1]), d2 = op_sub(u[2], p[2]);
-  v[1] = op_fma(d2, d2, op_fma(d1, d1, op_mul(d0, d0)));
-  v[2] = op_fma(u[2], u[2], op_fma(u[1], u[1], op_mul(u[0], u[0])));
-  const bool ok = isfinite(rho) && rho > 0.0 && isfinite(u[0]) && isfinite(u[1]) && isfinite(u[2]);
-  v[3] = ok ? 0.0 : 1.0;
+__device__ __forceinline__ double warp_terms_f64(const NodeTerms<T>& t, bool active, double rho0) {
+  double q[4] = {0.0, 0.0, 0.0, 0.0};
+  if (active) {
+    const double rho = rho0 + double(t.drho);
+    const double u[3] = {double(t.u[0]), double(t.u[1]), double(t.u[2])};
+    const double d0 = op_sub(u[0], double(t.p[0])), d1 = op_sub(u[1], double(t.p[1])), d2 = op_sub(u[2], double(t.p[2]));
+    q[0] = double(t.drho);
+    q[1] = op_fma(d2, d2, op_fma(d1, d1, op_mul(d0, d0)));
+    q[2] = op_fma(u[2], u[2], op_fma(u[1], u[1], op_mul(u[0], u[0])));
+    const bool ok = isfinite(rho) && rho > 0.0 && isfinite(u[0]) && isfinite(u[1]) && isfinite(u[2]);
+    q[3] = ok ? 0.0 : 1.0;
+  }
+  return warp_sum4(q[0], q[1], q[2], q[3]);
+}
+
+// hi + lo of (a - b)^2 for a difference taken exactly (TwoSum), to about 2^-47
+__device__ __forceinline__ fpair square_diff(float a, float b) {
+  const float d = __fsub_rn(a, b);
+  const float bb = __fsub_rn(d, a);
+  const float e = __fsub_rn(__fsub_rn(a, __fsub_rn(d, bb)), __fadd_rn(b, bb));
+  const float h = __fmul_rn(d, d);
+  return {h, __fmaf_rn(__fmul_rn(2.0f, d), e, __fmaf_rn(d, d, -h))};
+}
+__device__ __forceinline__ fpair square(float a) {
+  const float h = __fmul_rn(a, a);
+  return {h, __fmaf_rn(a, a, -h)};
+}
+
+// Block sums of the residual reductions over the active threads of block `blk` (nodes
+// blk*256 .. of N), into out[4]; every thread of the block takes part. The snapshot takes
+// the velocities. Float lattices form the node terms and
+// the warp sums as float pairs (about 48 bits): in double they were 45 FP64 instructions
+// per warp, about 850 SM cycles against 260 for the memory traffic of its nodes. The
+// velocities are scaled by 2^32 so that squares neither overflow nor lose their low
+// parts; a warp with a value outside the range that this covers (|u| >= 2^26, a density
+// deviation beyond 2^64, not-a-number, or a largest velocity or change below 2^-72 that
+// is not zero) forms its sums in double. So do FP64 lattices. The warp results are
+// added in double in either case.
+template <typename T>
+__device__ __forceinline__ void block_terms(const NodeTerms<T>& t, uint32_t N, uint32_t blk, double rho0,
+                                            float neg_rho0, T* snap, double* out) {
+  constexpr int WARPS = SWEEP_THREADS / 32;
+  const uint32_t cell = blk * SWEEP_THREADS + threadIdx.x;
+  const uint32_t nodes = N - blk * SWEEP_THREADS < SWEEP_THREADS ? N - blk * SWEEP_THREADS : SWEEP_THREADS;
+  const bool active = threadIdx.x < nodes;
+  __shared__ double sums[WARPS][4];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if constexpr (std::is_same<T, double>::value) {
+    const double k = warp_terms_f64(t, active, rho0);
+    if ((lane & 7) == 0) sums[warp][lane >> 3] = k;
+    __syncthreads();
+    if (active) store_snapshot(t, snap, N, cell);
+    if (warp == 0) {
+      double v = block_sum_rows(sums[lane >> 2][lane & 3]);
+      if (lane == 0) v = op_fma(rho0, double(nodes), v);
+      if (lane < 4) out[lane] = v;
+    }
+  } else {
+    __shared__ fpair pairs[WARPS][4];
+    __shared__ bool in_pairs[WARPS];
+    float u[3], p[3], drho = 0.0f;
+    bool ok = true, range = true;
+    float big = 0.0f, step = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) u[i] = p[i] = 0.0f;
+    if (active) {
+      drho = t.drho;
+      range = fabsf(drho) < 0x1p64f;
+      ok = drho > neg_rho0 && drho < INFINITY;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        ok = ok && fabsf(t.u[i]) < INFINITY;
+        range = range && fabsf(t.u[i]) < 0x1p26f && fabsf(t.p[i]) < 0x1p26f;
+        u[i] = __fmul_rn(t.u[i], 0x1p32f);
+        p[i] = __fmul_rn(t.p[i], 0x1p32f);
+        big = fmaxf(big, fabsf(u[i]));
+        step = fmaxf(step, fabsf(__fsub_rn(u[i], p[i])));
+      }
+    }
+    // non-negative floats order as their bits do
+    const uint32_t bits_u = __reduce_max_sync(0xffffffffu, __float_as_uint(big));
+    const uint32_t bits_d = __reduce_max_sync(0xffffffffu, __float_as_uint(step));
+    const uint32_t least = __float_as_uint(0x1p-40f);
+    if (__all_sync(0xffffffffu, range) && (bits_u == 0u || bits_u >= least) && (bits_d == 0u || bits_d >= least)) {
+      const uint32_t bad = __popc(__ballot_sync(0xffffffffu, !ok));
+      const fpair d2 = sum_of(sum_of(square_diff(u[0], p[0]), square_diff(u[1], p[1])), square_diff(u[2], p[2]));
+      const fpair u2 = sum_of(sum_of(square(u[0]), square(u[1])), square(u[2]));
+      const fpair k = warp_sum4(fpair{drho, 0.0f}, d2, u2, fpair{0.0f, 0.0f});
+      if ((lane & 7) == 0) pairs[warp][lane >> 3] = lane == 24 ? fpair{float(bad), 0.0f} : k;
+      if (lane == 0) in_pairs[warp] = true;
+    } else {
+      const double k = warp_terms_f64(t, active, rho0);
+      if ((lane & 7) == 0) sums[warp][lane >> 3] = k;
+      if (lane == 0) in_pairs[warp] = false;
+    }
+    __syncthreads();
+    if (active) store_snapshot(t, snap, N, cell);
+    if (warp == 0) {
+      const int w = lane >> 2, j = lane & 3;
+      double v;
+      if (in_pairs[w]) {
+        v = double(pairs[w][j].hi) + double(pairs[w][j].lo);
+        if (j == 1 || j == 2) v = op_mul(v, 0x1p-64);
+      } else {
+        v = sums[w][j];
+      }
+      v = block_sum_rows(v);
+      if (lane == 0) v = op_fma(rho0, double(nodes), v);
+      if (lane < 4) out[lane] = v;
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------------
@@ -841,7 +936,7 @@ __device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk) {
   using T = typename ComputeOf<S>::T;
   const uint32_t cell = blk * SWEEP_THREADS + threadIdx.x;
   const bool active = cell < a.N;
-  double red[4] = {0.0, 0.0, 0.0, 0.0};
+  NodeTerms<T> terms = {};
   if (active) {
     const uint32_t q1 = fdiv(a.div_nx, cell);
     const uint32_t x = cell - q1 * a.nx;
@@ -923,7 +1018,7 @@ __device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk) {
           mp.ux = mp.jx * inv;
           mp.uy = mp.jy * inv;
           mp.uz = mp.jz * inv;
-          residual_terms(mp, ref_rho<S>(a.rho0), static_cast<T*>(a.snap), a.N, cell, red);
+          terms = residual_terms(mp, static_cast<T*>(a.snap), a.N, cell);
         }
         m.jx += tforce_of<T>(a, 0);
         m.jy += tforce_of<T>(a, 1);
@@ -932,10 +1027,10 @@ __device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk) {
         m.uy = m.jy * inv;
         m.uz = m.jz * inv;
       } else if constexpr (RESID) {
-        residual_terms(m, ref_rho<S>(a.rho0), static_cast<T*>(a.snap), a.N, cell, red);
+        terms = residual_terms(m, static_cast<T*>(a.snap), a.N, cell);
       }
     } else if constexpr (RESID) {
-      residual_terms(m, ref_rho<S>(a.rho0), static_cast<T*>(a.snap), a.N, cell, red);
+      terms = residual_terms(m, static_cast<T*>(a.snap), a.N, cell);
     }
     if (!solid) collide<std::is_same<S, float>::value>(h, m, omega_of<T>(a), a.mom_coef);
     static_for<0, Q>([&](auto kc) {
@@ -955,7 +1050,8 @@ __device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk) {
       }
     });
   }
-  if constexpr (RESID) block_sum4(red, a.partials + 4ull * blk);
+  if constexpr (RESID)
+    block_terms(terms, a.N, blk, ref_rho<S>(a.rho0), a.neg_rho0, static_cast<T*>(a.snap), a.partials + 4ull * blk);
 }
 
 // Resident 256-thread blocks per SM each sweep variant is compiled for (the register
@@ -1482,21 +1578,21 @@ __global__ void __launch_bounds__(SWEEP_THREADS, (SweepOccupancy<S, RESID, true,
 // SWAPPED: the state holds f_k in slot -k (an AA lattice after a local step).
 template <typename S, bool SWAPPED = false>
 __global__ void __launch_bounds__(SWEEP_THREADS)
-    state_reduce_kernel(const S* __restrict__ src, uint32_t N, double rho0, void* snap, double* partials) {
+    state_reduce_kernel(const S* __restrict__ src, uint32_t N, double rho0, float neg_rho0, void* snap,
+                        double* partials) {
   using T = typename ComputeOf<S>::T;
   const uint32_t cell = blockIdx.x * SWEEP_THREADS + threadIdx.x;
-  double red[4] = {0.0, 0.0, 0.0, 0.0};
+  NodeTerms<T> terms = {};
   if (cell < N) {
     T h[Q];
     static_for<0, Q>([&](auto kc) {
       constexpr int k = decltype(kc)::value;
       h[k] = Storage<S>::load(src + size_t(SWAPPED ? opp(k) : k) * N + cell);
     });
-    const double ref = ref_rho<S>(rho0);
-    const Moments<T> m = moments(h, T(ref));
-    residual_terms(m, ref, static_cast<T*>(snap), N, cell, red);
+    const Moments<T> m = moments(h, T(ref_rho<S>(rho0)));
+    terms = residual_terms(m, static_cast<T*>(snap), N, cell);
   }
-  block_sum4(red, partials + 4ull * blockIdx.x);
+  block_terms(terms, N, blockIdx.x, ref_rho<S>(rho0), neg_rho0, static_cast<T*>(snap), partials + 4ull * blockIdx.x);
 }
 
 template <typename S>
@@ -1621,11 +1717,12 @@ cudaError_t launch_macros_impl(const void* src, uint32_t N, double rho0, void* r
 template <typename S>
 cudaError_t launch_state_reduce_impl(const void* src, uint32_t N, double rho0, void* snap, double* partials,
                                      bool swapped, cudaStream_t s) {
+  const float nr = floor_neg(rho0);
   if (swapped)
-    state_reduce_kernel<S, true><<<sweep_blocks(N), SWEEP_THREADS, 0, s>>>(static_cast<const S*>(src), N, rho0,
+    state_reduce_kernel<S, true><<<sweep_blocks(N), SWEEP_THREADS, 0, s>>>(static_cast<const S*>(src), N, rho0, nr,
                                                                            snap, partials);
   else
-    state_reduce_kernel<S, false><<<sweep_blocks(N), SWEEP_THREADS, 0, s>>>(static_cast<const S*>(src), N, rho0,
+    state_reduce_kernel<S, false><<<sweep_blocks(N), SWEEP_THREADS, 0, s>>>(static_cast<const S*>(src), N, rho0, nr,
                                                                             snap, partials);
   return cudaGetLastError();
 }

@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
+#include <cmath>
 #include <cstdint>
 
 namespace lbm {
@@ -31,6 +32,12 @@ __device__ __forceinline__ uint32_t fdiv(const FastDiv& f, uint32_t n) {
   return (t + ((n - t) >> f.s1)) >> f.s2;
 }
 #endif
+
+// Largest float not above -rho0: for a float drho, rho0 + drho > 0 exactly if drho > it.
+inline float floor_neg(double rho0) {
+  const float f = float(-rho0);
+  return double(f) > -rho0 ? std::nextafter(f, -INFINITY) : f;
+}
 
 // One boundary-face node as the sweep reads it. Velocity face: the prescribed velocity
 // in double and float, and 1 / (1 - u.n) for the density relation (n = inward normal),
@@ -63,10 +70,11 @@ struct SweepArgs {
   double rho0;
   double omega;       // 1 / tau
   float rho0f, omegaf;
+  float neg_rho0;     // floor_neg(rho0)
   float mom_coef[2][2];  // omegaf / 6 and omegaf / 12 as hi + lo float pairs
   FaceBC face[6];
   void* snap;         // residual steps: [3][N] velocity snapshot in the compute type
-  double* partials;   // residual steps: [blocks][4] per-block sums
+  double* partials;   // residual steps: [blocks][4] per-block sums, then [groups][4] of the fold
   const uint32_t* links;  // optional [N] geometry words (nullptr: no geometry), see below
   uint32_t forced;        // nonzero: a body force acts (eq. gravity)
   double force[3];        // F: momentum the collision adds per step
@@ -119,9 +127,16 @@ struct BatchChunk {
 };
 
 constexpr int SWEEP_THREADS = 256;
-constexpr int REDUCE_THREADS = 1024;
+// Final fold of the partial sums: one block of FOLD_THREADS folds FOLD_ROWS rows.
+constexpr int FOLD_THREADS = 256;
+constexpr uint32_t FOLD_ROWS = 1024;
 
 inline uint32_t sweep_blocks(uint32_t N) { return (N + SWEEP_THREADS - 1) / SWEEP_THREADS; }
+// groups of the fold of `nblocks` rows (19 N < 2^32, so nblocks < 2^20 and one more level
+// of FOLD_ROWS rows folds the groups)
+__host__ __device__ inline uint32_t fold_groups(uint32_t nblocks) { return (nblocks + FOLD_ROWS - 1) / FOLD_ROWS; }
+// rows of a partial-sum buffer: the sweep's blocks, then the fold's groups
+inline uint32_t partial_rows(uint32_t nblocks) { return nblocks + fold_groups(nblocks); }
 
 // mode: 0 A/B pull, 1 AA gather-scatter step, 2 AA in-place step (see kernels.cuh)
 template <typename S> cudaError_t launch_sweep(const SweepArgs& a, bool resid, int mode, cudaStream_t s);
@@ -131,7 +146,9 @@ template <typename S> cudaError_t launch_macros(const void* src, uint32_t N, dou
                                                 void* u, bool swapped, cudaStream_t s);
 template <typename S> cudaError_t launch_state_reduce(const void* src, uint32_t N, double rho0,
                                                       void* snap, double* partials, bool swapped, cudaStream_t s);
-cudaError_t launch_final_reduce(const double* partials, uint32_t nblocks, double* out, cudaStream_t s);
+// partials: partial_rows(nblocks) rows, the first nblocks of them summed into out[4];
+// ticket: a device word that is zero between folds
+cudaError_t launch_final_reduce(double* partials, uint32_t nblocks, double* out, uint32_t* ticket, cudaStream_t s);
 // next_chunk: a device counter that is zero when the launch starts (the caller clears
 // it in stream order before every launch); each CTA draws chunks from it until the
 // table is exhausted

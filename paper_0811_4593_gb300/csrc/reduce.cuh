@@ -1,30 +1,80 @@
-// reduce.cuh -- fixed-order fold of per-block partial sums, shared by the single-lattice
-// and the batched final reductions so that a lattice reduces to the same bits in both.
+// reduce.cuh -- fixed-order sums of the residual reductions (mass, |du|^2, |u|^2 and a
+// bad-node count), shared by the sweeps, the single-lattice and the batched final folds
+// so that a lattice reduces to the same bits in all of them.
+//
+// The FP64 pipe issues one warp instruction in about 19 SM cycles (527 G thread
+// operations per second on 152 SMs), so the sums are arranged to issue few of them.
 #pragma once
 #include "lbm_internal.h"
 
 namespace lbm {
 
-// One block of REDUCE_THREADS folds partials[nblocks][4] into out[4]: thread t sums
-// blocks t, t + REDUCE_THREADS, ... in ascending order, then a fixed pairwise tree over
-// the threads. The order depends only on nblocks.
-__device__ __forceinline__ void fold_partials(const double* __restrict__ partials, uint32_t nblocks,
-                                              double* __restrict__ out) {
-  __shared__ double s[4][REDUCE_THREADS];
+// An unevaluated float sum hi + lo (lo below half an ulp of hi after each accumulation
+// of hi; about 48 bits).
+struct fpair {
+  float hi, lo;
+};
+
+__device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ fpair shfl_xor(fpair v, int o) {
+  return {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+}
+__device__ __forceinline__ double sum_of(double a, double b) { return __dadd_rn(a, b); }
+// Sum of two pairs: the high parts by Knuth's TwoSum (error-free), the low parts and the
+// error by rounded float additions.
+__device__ __forceinline__ fpair sum_of(fpair a, fpair b) {
+  const float s = __fadd_rn(a.hi, b.hi);
+  const float t = __fsub_rn(s, a.hi);
+  const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, t)), __fsub_rn(b.hi, t));
+  return {s, __fadd_rn(__fadd_rn(a.lo, b.lo), e)};
+}
+
+// Warp totals of four quantities: lane l returns the total of quantity l / 8. The first
+// two steps halve what a lane still carries instead of reducing four values over five
+// steps each, so a warp issues 6 additions in place of 20.
+template <typename V>
+__device__ __forceinline__ V warp_sum4(V q0, V q1, V q2, V q3) {
+  const bool up = threadIdx.x & 16, up2 = threadIdx.x & 8;
+  const V k0 = sum_of(up ? q2 : q0, shfl_xor(up ? q0 : q2, 16));
+  const V k1 = sum_of(up ? q3 : q1, shfl_xor(up ? q1 : q3, 16));
+  V k = sum_of(up2 ? k1 : k0, shfl_xor(up2 ? k0 : k1, 8));
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) k = sum_of(k, shfl_xor(k, o));
+  return k;
+}
+
+// Totals over the 8 warps of a 256-thread block from one row of four doubles per warp
+// (lane l of the first warp holds row l / 4, quantity l % 4); valid in its lanes 0..3.
+__device__ __forceinline__ double block_sum_rows(double v) {
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) v = sum_of(v, shfl_xor(v, o));
+  return v;
+}
+
+// FOLD_THREADS threads fold `count` <= FOLD_ROWS rows of four doubles into out[4]:
+// thread t adds rows t, t + FOLD_THREADS, ... in ascending order, then the warp and
+// block sums above. The order depends only on `count`. Ends with a block barrier behind
+// the write of out.
+__device__ __forceinline__ void fold_rows(const double* rows, uint32_t count, double* out) {
+  __shared__ double warp_rows[FOLD_THREADS / 32][4];
   double v[4] = {0.0, 0.0, 0.0, 0.0};
-  for (uint32_t b = threadIdx.x; b < nblocks; b += REDUCE_THREADS)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] += partials[4ull * b + j];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) s[j][threadIdx.x] = v[j];
-  __syncthreads();
-  for (int w = REDUCE_THREADS / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) s[j][threadIdx.x] += s[j][threadIdx.x + w];
-    __syncthreads();
+  for (uint32_t b = threadIdx.x; b < count; b += FOLD_THREADS) {
+    const double2 x = __ldcg(reinterpret_cast<const double2*>(rows) + 2ull * b);
+    const double2 y = __ldcg(reinterpret_cast<const double2*>(rows) + 2ull * b + 1);
+    v[0] += x.x;
+    v[1] += x.y;
+    v[2] += y.x;
+    v[3] += y.y;
   }
-  if (threadIdx.x < 4) out[threadIdx.x] = s[threadIdx.x][0];
+  const double k = warp_sum4(v[0], v[1], v[2], v[3]);
+  const int lane = threadIdx.x & 31;
+  if ((lane & 7) == 0) warp_rows[threadIdx.x >> 5][lane >> 3] = k;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const double s = block_sum_rows(warp_rows[lane >> 2][lane & 3]);
+    if (lane < 4) out[lane] = s;
+  }
+  __syncthreads();
 }
 
 }  // namespace lbm

@@ -5,6 +5,7 @@
 
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -47,8 +48,9 @@ struct lbm_ctx {
   int cur = 0;  // A/B: buf[cur] holds the current post-collision state
   void* snap = nullptr;
   double* partials = nullptr;
-  double* dred = nullptr;
-  uint32_t* derr = nullptr;  // device error word of the sweeps (SweepArgs::err)
+  double* dred = nullptr;    // reduction results [4], and behind them
+  uint32_t* derr = nullptr;  // the error word of the sweeps (SweepArgs::err)
+  uint32_t* dticket = nullptr;  // and the fold's ticket
   cudaStream_t stream = nullptr;
   int64_t steps = 0, launches = 0, device_bytes = 0;
   std::string err = "no error";
@@ -297,7 +299,7 @@ lbm_status ensure_reduction_buffers(lbm_ctx* ctx) {
   const size_t snap_bytes = 3ull * ctx->N * compute_bytes(ctx->prec);
   void* snap = ctx_alloc(ctx, snap_bytes);
   if (!snap) return fail(ctx, LBM_ERR_OOM, "allocation of %zu bytes for the velocity snapshot failed", snap_bytes);
-  const size_t part_bytes = 4ull * lbm::sweep_blocks(ctx->N) * sizeof(double);
+  const size_t part_bytes = 4ull * lbm::partial_rows(lbm::sweep_blocks(ctx->N)) * sizeof(double);
   void* part = ctx_alloc(ctx, part_bytes);
   if (!part) return fail(ctx, LBM_ERR_OOM, "allocation of %zu bytes for reduction partials failed", part_bytes);
   LBM_CUDA(ctx, cudaMemsetAsync(snap, 0, snap_bytes, ctx->stream), "clearing the velocity snapshot");
@@ -315,33 +317,45 @@ lbm_status settle(lbm_ctx* ctx) {
   return LBM_OK;
 }
 
-// Final fold of the partial sums and the host-side residual.
-// Reads (and clears) the sweeps' device error word after synchronising the stream: a
-// sweep that gave up waiting for its staged loads left results that are not valid.
-lbm_status check_device_error(lbm_ctx* ctx) {
-  LBM_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "stream synchronisation");
-  if (!ctx->derr) return LBM_OK;
-  uint32_t v = 0;
-  LBM_CUDA(ctx, cudaMemcpyAsync(&v, ctx->derr, sizeof v, cudaMemcpyDeviceToHost, ctx->stream), "reading the error word");
-  LBM_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "reading the error word");
+// What an error word read from the device says: a sweep that gave up waiting for its
+// staged loads left results that are not valid. Clears a set word.
+lbm_status report_device_error(lbm_ctx* ctx, uint32_t v) {
   if (v == 0) return LBM_OK;
   LBM_CUDA(ctx, cudaMemsetAsync(ctx->derr, 0, sizeof v, ctx->stream), "clearing the error word");
   return fail(ctx, LBM_ERR_CUDA,
               "a sweep gave up waiting for its staged row copies (device error word 0x%x): the state is not valid", v);
 }
 
+// Synchronises the stream, then reads (and clears) the sweeps' device error word.
+lbm_status check_device_error(lbm_ctx* ctx) {
+  LBM_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "stream synchronisation");
+  if (!ctx->derr) return LBM_OK;
+  uint32_t v = 0;
+  LBM_CUDA(ctx, cudaMemcpyAsync(&v, ctx->derr, sizeof v, cudaMemcpyDeviceToHost, ctx->stream), "reading the error word");
+  LBM_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "reading the error word");
+  return report_device_error(ctx, v);
+}
+
+// Final fold of the partial sums and the host-side residual. The results and the error
+// word lie together and come back in one copy.
+
 lbm_status finish_reduction(lbm_ctx* ctx, double* residual, double* mass) {
-  LBM_CUDA(ctx, lbm::launch_final_reduce(ctx->partials, lbm::sweep_blocks(ctx->N), ctx->dred, ctx->stream),
+  LBM_CUDA(ctx, lbm::launch_final_reduce(ctx->partials, lbm::sweep_blocks(ctx->N), ctx->dred, ctx->dticket, ctx->stream),
            "final reduction launch");
   ctx->launches += 1;
-  double h[4];
-  LBM_CUDA(ctx, cudaMemcpyAsync(h, ctx->dred, sizeof h, cudaMemcpyDeviceToHost, ctx->stream), "reading reductions");
+  struct {
+    double red[4];
+    uint32_t err;
+  } r;
+  LBM_CUDA(ctx, cudaMemcpyAsync(&r, ctx->dred, offsetof(decltype(r), err) + sizeof r.err, cudaMemcpyDeviceToHost, ctx->stream),
+           "reading reductions");
   LBM_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "synchronising after reductions");
-  if (lbm_status st = check_device_error(ctx); st != LBM_OK) return st;
-  const double r = h[2] > 0.0 ? std::sqrt(h[1]) / std::sqrt(h[2]) : std::sqrt(h[1]);
-  if (residual) *residual = r;
+  if (lbm_status st = report_device_error(ctx, r.err); st != LBM_OK) return st;
+  const double* h = r.red;
+  const double res = h[2] > 0.0 ? std::sqrt(h[1]) / std::sqrt(h[2]) : std::sqrt(h[1]);
+  if (residual) *residual = res;
   if (mass) *mass = h[0];
-  if (h[3] != 0.0 || !std::isfinite(h[0]) || !std::isfinite(r))
+  if (h[3] != 0.0 || !std::isfinite(h[0]) || !std::isfinite(res))
     return fail(ctx, LBM_ERR_DIVERGED, "diverged: %.0f nodes with non-finite or non-positive density or "
                 "non-finite velocity (mass %g)", h[3], h[0]);
   return LBM_OK;
@@ -402,12 +416,13 @@ lbm_status lbm_create_scheme(int nx, int ny, int nz, double tau, const lbm_face_
     if (!ctx->buf[b]) return bail(fail(ctx, LBM_ERR_OOM, "allocation of %zu bytes for populations failed", pop_bytes));
   }
   if (scheme == LBM_SCHEME_AA) ctx->buf[1] = ctx->buf[0];
-  ctx->dred = static_cast<double*>(ctx_alloc(ctx, 4 * sizeof(double)));
+  const size_t red_bytes = 4 * sizeof(double) + 2 * sizeof(uint32_t);
+  ctx->dred = static_cast<double*>(ctx_alloc(ctx, red_bytes));
   if (!ctx->dred) return bail(fail(ctx, LBM_ERR_OOM, "allocation of the reduction result failed"));
-  ctx->derr = static_cast<uint32_t*>(ctx_alloc(ctx, sizeof(uint32_t)));
-  if (!ctx->derr) return bail(fail(ctx, LBM_ERR_OOM, "allocation of the error word failed"));
-  e = cudaMemsetAsync(ctx->derr, 0, sizeof(uint32_t), ctx->stream);
-  if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "clearing the error word"));
+  ctx->derr = reinterpret_cast<uint32_t*>(ctx->dred + 4);
+  ctx->dticket = ctx->derr + 1;
+  e = cudaMemsetAsync(ctx->dred, 0, red_bytes, ctx->stream);
+  if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "clearing the reduction result and the error word"));
 
   lbm::SweepArgs& a = ctx->args;
   a.nx = nx; a.ny = ny; a.nz = nz; a.N = ctx->N;
@@ -421,6 +436,7 @@ lbm_status lbm_create_scheme(int nx, int ny, int nz, double tau, const lbm_face_
   a.rho0 = rho0;
   a.omega = 1.0 / tau;
   a.rho0f = float(rho0);
+  a.neg_rho0 = lbm::floor_neg(rho0);
   a.omegaf = float(1.0 / tau);
   // 3 omega w_i of the BGK update's momentum term for the float sweep, as hi + lo
   // floats of omegaf / 6 (axis) and omegaf / 12 (diagonal): with a single rounded

@@ -15,11 +15,15 @@
 
 namespace {
 
-// 65,536 blocks of 256 nodes: lattices up to 16,777,216 nodes (256^3); 2 MiB per device.
+// 65,536 blocks of 256 nodes: lattices up to 16,777,216 nodes (256^3); 2 MiB per device,
+// and the rows and the ticket of the final fold behind them.
 constexpr uint32_t kStaticBlocks = 65536;
+constexpr uint32_t kStaticRows = kStaticBlocks + kStaticBlocks / lbm::FOLD_ROWS;
 constexpr int kMaxDevices = 64;
 
-__device__ __align__(256) double g_static_partials[4 * kStaticBlocks];
+// the last double holds the fold's ticket (zero when the library is loaded, and again
+// after every fold)
+__device__ __align__(256) double g_static_partials[4 * kStaticRows + 1];
 
 std::mutex g_setup_mu;
 void* g_partials_addr[kMaxDevices] = {};
@@ -81,19 +85,20 @@ extern "C" LBM_API lbm_status lbm_reduce_state_static(const void* populations, i
   switch (prec) {
     case LBM_F64:
       lbm::state_reduce_kernel<double><<<blocks, lbm::SWEEP_THREADS, 0, s>>>(
-          static_cast<const double*>(populations), N, rho0, velocity_snapshot, partials);
+          static_cast<const double*>(populations), N, rho0, lbm::floor_neg(rho0), velocity_snapshot, partials);
       break;
     case LBM_F32:
       lbm::state_reduce_kernel<float><<<blocks, lbm::SWEEP_THREADS, 0, s>>>(
-          static_cast<const float*>(populations), N, rho0, velocity_snapshot, partials);
+          static_cast<const float*>(populations), N, rho0, lbm::floor_neg(rho0), velocity_snapshot, partials);
       break;
     default:
       lbm::state_reduce_kernel<__half><<<blocks, lbm::SWEEP_THREADS, 0, s>>>(
-          static_cast<const __half*>(populations), N, rho0, velocity_snapshot, partials);
+          static_cast<const __half*>(populations), N, rho0, lbm::floor_neg(rho0), velocity_snapshot, partials);
       break;
   }
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = lbm::launch_final_reduce(partials, blocks, sums, s);
+  uint32_t* ticket = reinterpret_cast<uint32_t*>(partials + 4ull * kStaticRows);
+  if (e == cudaSuccess) e = lbm::launch_final_reduce(partials, blocks, sums, ticket, s);
   if (e != cudaSuccess) {
     char buf[256];
     snprintf(buf, sizeof buf, "lbm_reduce_state_static: launch failed: %s", cudaGetErrorString(e));
