@@ -14,6 +14,7 @@
 #include <utility>
 
 #include "d3q19.cuh"
+#include "fixed64.cuh"
 #include "lbm_internal.h"
 #include "reduce.cuh"
 
@@ -915,6 +916,100 @@ __device__ __forceinline__ void block_terms(const NodeTerms<T>& t, uint32_t N, u
   }
 }
 
+// Density and velocity of an FP64 node from its fixed-point sums (each rounded once to
+// double; FORCE is added to the momentum).
+__device__ __forceinline__ Moments<double> moments_of(const FixedSums& q, const FixedArgs& fx, const double* force) {
+  double s[4];
+  fixed_to_double(q, fx, s);
+  if (force) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) s[1 + i] += force[i];
+  }
+  Moments<double> m;
+  m.drho = m.rho = s[0];
+  m.jx = s[1];
+  m.jy = s[2];
+  m.jz = s[3];
+  m.inv = 1.0 / m.rho;
+  m.ux = op_mul(m.jx, m.inv);
+  m.uy = op_mul(m.jy, m.inv);
+  m.uz = op_mul(m.jz, m.inv);
+  return m;
+}
+__device__ __forceinline__ FixedSums fixed_sums_of(const double (&h)[Q], const FixedArgs& fx, int64_t (&f)[Q]) {
+  static_for<0, Q>([&](auto kc) { f[decltype(kc)::value] = fixed_in(h[decltype(kc)::value], fx); });
+  return fixed_sums(f);
+}
+
+// Moments of a stored node for the read-outs: FP64 in fixed point where the node allows
+// it (33 integer additions in place of 37 FP64 ones), else as in the sweep.
+template <typename S, typename T>
+__device__ __forceinline__ Moments<T> stored_moments(const T (&h)[Q], double rho0, const FixedArgs& fx) {
+  if constexpr (std::is_same<T, double>::value) {
+    if (fx.on && fixed_in_range(h, fx)) {
+      int64_t f[Q];
+      return moments_of(fixed_sums_of(h, fx, f), fx, nullptr);
+    }
+  }
+  return moments(h, T(ref_rho<S>(rho0)));
+}
+
+// Moments, residual terms and relaxation of one node on its closed populations. FP64
+// nodes whose populations lie in the windows of fixed64.cuh are relaxed there; with
+// RESID their density and velocity are the fixed-point sums rounded to double.
+template <typename S, bool RESID, bool GEOM, typename T>
+__device__ __forceinline__ void relax_node(const SweepArgs& a, T (&h)[Q], uint32_t cell, bool solid, NodeTerms<T>& terms) {
+  T* snap = static_cast<T*>(a.snap);
+  if constexpr (std::is_same<T, double>::value) {
+    if (a.fx.on && !solid && fixed_in_range(h, a.fx)) {
+      int64_t f[Q];
+      FixedSums q = fixed_sums_of(h, a.fx, f);
+      if constexpr (RESID)
+        terms = residual_terms(moments_of(q, a.fx, GEOM && a.forced ? a.force : nullptr), snap, a.N, cell);
+      if constexpr (GEOM) {
+        if (a.forced) {
+          q.x += a.fx.force[0];
+          q.y += a.fx.force[1];
+          q.z += a.fx.force[2];
+        }
+      }
+      fixed_relax(f, q, a.fx, h);
+      return;
+    }
+  }
+  Moments<T> m;
+  if constexpr (GEOM && std::is_same<S, float>::value) m = moments_compensated(h, rho0_of<T>(a));
+  else m = moments(h, rho0_of<T>(a));
+  if constexpr (GEOM) {
+    if (a.forced && !solid) {
+      // eq. gravity: the collision relaxes toward the equilibrium at u + tau F / rho
+      // and so adds F to the momentum; the residual sees the stored velocity
+      const T inv = T(1) / m.rho;
+      if constexpr (RESID) {
+        Moments<T> mp = m;
+        mp.jx += force_of<T>(a, 0);
+        mp.jy += force_of<T>(a, 1);
+        mp.jz += force_of<T>(a, 2);
+        mp.ux = mp.jx * inv;
+        mp.uy = mp.jy * inv;
+        mp.uz = mp.jz * inv;
+        terms = residual_terms(mp, snap, a.N, cell);
+      }
+      m.jx += tforce_of<T>(a, 0);
+      m.jy += tforce_of<T>(a, 1);
+      m.jz += tforce_of<T>(a, 2);
+      m.ux = m.jx * inv;
+      m.uy = m.jy * inv;
+      m.uz = m.jz * inv;
+    } else if constexpr (RESID) {
+      terms = residual_terms(m, snap, a.N, cell);
+    }
+  } else if constexpr (RESID) {
+    terms = residual_terms(m, snap, a.N, cell);
+  }
+  if (!solid) collide<std::is_same<S, float>::value>(h, m, omega_of<T>(a), a.mom_coef);
+}
+
 // ---------------------------------------------------------------------------------
 // The fused time step: pull stream, classify, close, collide, store.
 // ---------------------------------------------------------------------------------
@@ -1002,37 +1097,7 @@ __device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk) {
     } else {
       if (code != 0) apply_boundary(code, a, x, y, z, h);
     }
-    Moments<T> m;
-    if constexpr (GEOM && std::is_same<S, float>::value) m = moments_compensated(h, rho0_of<T>(a));
-    else m = moments(h, rho0_of<T>(a));
-    if constexpr (GEOM) {
-      if (a.forced && !solid) {
-        // eq. gravity: the collision relaxes toward the equilibrium at u + tau F / rho
-        // and so adds F to the momentum; the residual sees the stored velocity
-        const T inv = T(1) / m.rho;
-        if constexpr (RESID) {
-          Moments<T> mp = m;
-          mp.jx += force_of<T>(a, 0);
-          mp.jy += force_of<T>(a, 1);
-          mp.jz += force_of<T>(a, 2);
-          mp.ux = mp.jx * inv;
-          mp.uy = mp.jy * inv;
-          mp.uz = mp.jz * inv;
-          terms = residual_terms(mp, static_cast<T*>(a.snap), a.N, cell);
-        }
-        m.jx += tforce_of<T>(a, 0);
-        m.jy += tforce_of<T>(a, 1);
-        m.jz += tforce_of<T>(a, 2);
-        m.ux = m.jx * inv;
-        m.uy = m.jy * inv;
-        m.uz = m.jz * inv;
-      } else if constexpr (RESID) {
-        terms = residual_terms(m, static_cast<T*>(a.snap), a.N, cell);
-      }
-    } else if constexpr (RESID) {
-      terms = residual_terms(m, static_cast<T*>(a.snap), a.N, cell);
-    }
-    if (!solid) collide<std::is_same<S, float>::value>(h, m, omega_of<T>(a), a.mom_coef);
+    relax_node<S, RESID, GEOM>(a, h, cell, solid, terms);
     static_for<0, Q>([&](auto kc) {
       constexpr int k = decltype(kc)::value;
       if constexpr (MODE == STREAM_AB) {
@@ -1072,7 +1137,7 @@ struct SweepOccupancy {
 };
 template <bool RESID, bool BATCHED, int MODE, bool GEOM>
 struct SweepOccupancy<double, RESID, BATCHED, MODE, GEOM> {
-  static constexpr int blocks = (RESID && BATCHED) || MODE == 1 || GEOM ? 2 : 3;
+  static constexpr int blocks = RESID || MODE == 1 || GEOM ? 2 : 3;
 };
 
 template <typename S, bool RESID, int MODE, bool GEOM>
@@ -1578,8 +1643,8 @@ __global__ void __launch_bounds__(SWEEP_THREADS, (SweepOccupancy<S, RESID, true,
 // SWAPPED: the state holds f_k in slot -k (an AA lattice after a local step).
 template <typename S, bool SWAPPED = false>
 __global__ void __launch_bounds__(SWEEP_THREADS)
-    state_reduce_kernel(const S* __restrict__ src, uint32_t N, double rho0, float neg_rho0, void* snap,
-                        double* partials) {
+    state_reduce_kernel(const S* __restrict__ src, uint32_t N, double rho0, float neg_rho0,
+                        const __grid_constant__ FixedArgs fx, void* snap, double* partials) {
   using T = typename ComputeOf<S>::T;
   const uint32_t cell = blockIdx.x * SWEEP_THREADS + threadIdx.x;
   NodeTerms<T> terms = {};
@@ -1589,7 +1654,7 @@ __global__ void __launch_bounds__(SWEEP_THREADS)
       constexpr int k = decltype(kc)::value;
       h[k] = Storage<S>::load(src + size_t(SWAPPED ? opp(k) : k) * N + cell);
     });
-    const Moments<T> m = moments(h, T(ref_rho<S>(rho0)));
+    const Moments<T> m = stored_moments<S>(h, rho0, fx);
     terms = residual_terms(m, static_cast<T*>(snap), N, cell);
   }
   block_terms(terms, N, blockIdx.x, ref_rho<S>(rho0), neg_rho0, static_cast<T*>(snap), partials + 4ull * blockIdx.x);
@@ -1610,8 +1675,8 @@ __global__ void __launch_bounds__(SWEEP_THREADS) init_kernel(S* __restrict__ dst
 
 template <typename S, bool SWAPPED>
 __global__ void __launch_bounds__(SWEEP_THREADS)
-    macros_kernel(const S* __restrict__ src, uint32_t N, double rho0, typename ComputeOf<S>::T* rho,
-                  typename ComputeOf<S>::T* u) {
+    macros_kernel(const S* __restrict__ src, uint32_t N, double rho0, const __grid_constant__ FixedArgs fx,
+                  typename ComputeOf<S>::T* rho, typename ComputeOf<S>::T* u) {
   using T = typename ComputeOf<S>::T;
   const uint32_t cell = blockIdx.x * SWEEP_THREADS + threadIdx.x;
   if (cell >= N) return;
@@ -1620,7 +1685,7 @@ __global__ void __launch_bounds__(SWEEP_THREADS)
     constexpr int k = decltype(kc)::value;
     h[k] = Storage<S>::load(src + size_t(SWAPPED ? opp(k) : k) * N + cell);
   });
-  const Moments<T> m = moments(h, T(ref_rho<S>(rho0)));
+  const Moments<T> m = stored_moments<S>(h, rho0, fx);
   if (rho) rho[cell] = m.rho;
   if (u) {
     u[cell] = m.ux;
@@ -1701,29 +1766,31 @@ cudaError_t launch_init_impl(void* dst, uint32_t N, double rho0, cudaStream_t s)
   return cudaGetLastError();
 }
 
+// Fixed-point parameters of a read-out, which needs the density scale only.
+template <typename S>
+FixedArgs readout_fixed(double rho0) {
+  if (!std::is_same<S, double>::value) return FixedArgs{};
+  return make_fixed(rho0, 1.0, {0.0, 0.0, 0.0});
+}
+
 template <typename S>
 cudaError_t launch_macros_impl(const void* src, uint32_t N, double rho0, void* rho, void* u, bool swapped,
                                cudaStream_t s) {
   using T = typename ComputeOf<S>::T;
-  if (swapped)
-    macros_kernel<S, true><<<sweep_blocks(N), SWEEP_THREADS, 0, s>>>(static_cast<const S*>(src), N, rho0,
-                                                                     static_cast<T*>(rho), static_cast<T*>(u));
-  else
-    macros_kernel<S, false><<<sweep_blocks(N), SWEEP_THREADS, 0, s>>>(static_cast<const S*>(src), N, rho0,
-                                                                      static_cast<T*>(rho), static_cast<T*>(u));
+  const FixedArgs fx = readout_fixed<S>(rho0);
+  auto kernel = swapped ? macros_kernel<S, true> : macros_kernel<S, false>;
+  kernel<<<sweep_blocks(N), SWEEP_THREADS, 0, s>>>(static_cast<const S*>(src), N, rho0, fx, static_cast<T*>(rho),
+                                                   static_cast<T*>(u));
   return cudaGetLastError();
 }
 
 template <typename S>
 cudaError_t launch_state_reduce_impl(const void* src, uint32_t N, double rho0, void* snap, double* partials,
                                      bool swapped, cudaStream_t s) {
-  const float nr = floor_neg(rho0);
-  if (swapped)
-    state_reduce_kernel<S, true><<<sweep_blocks(N), SWEEP_THREADS, 0, s>>>(static_cast<const S*>(src), N, rho0, nr,
-                                                                           snap, partials);
-  else
-    state_reduce_kernel<S, false><<<sweep_blocks(N), SWEEP_THREADS, 0, s>>>(static_cast<const S*>(src), N, rho0, nr,
-                                                                            snap, partials);
+  const FixedArgs fx = readout_fixed<S>(rho0);
+  auto kernel = swapped ? state_reduce_kernel<S, true> : state_reduce_kernel<S, false>;
+  kernel<<<sweep_blocks(N), SWEEP_THREADS, 0, s>>>(static_cast<const S*>(src), N, rho0, floor_neg(rho0), fx, snap,
+                                                   partials);
   return cudaGetLastError();
 }
 

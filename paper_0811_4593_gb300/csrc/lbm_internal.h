@@ -56,6 +56,49 @@ struct FaceBC {
   FaceNode uni;
 };
 
+// Parameters of the fixed-point relaxation of FP64 lattices (fixed64.cuh), with S = 2^E.
+// Factors are (high, low) limbs of value 2^62.
+struct FixedArgs {
+  uint32_t on;        // 0: this lattice relaxes in double only
+  uint32_t e_in;      // biased exponent of S 2^-12
+  uint32_t e_out;     // (991 + E) << 20
+  int32_t keep[2];    // 1 - omega
+  int32_t w3[2];      // omega / 3
+  int32_t w[2];       // omega / 36
+  int64_t force[3];   // tau F in units of S 2^-64
+  double unit_in, unit_out;  // S 2^-64, S 2^-63
+};
+
+// The parameters for density scale rho0, omega and tau F. Off where a scale has no
+// normal double, where omega is below 2^-61 or where the force is not small.
+inline FixedArgs make_fixed(double rho0, double omega, const double (&tforce)[3]) {
+  FixedArgs fx{};
+  int e = 0;
+  const double m = std::frexp(rho0, &e);  // rho0 = m 2^e, 1/2 <= m < 1
+  e += m == 0.5 ? 1 : 2;                  // rho0 / 2^e in (1/8, 1/4]
+  if (e < -900 || e > 900 || !(omega > 0.0) || !(omega < 2.0)) return fx;
+  const int64_t w = int64_t(std::ldexp(omega, 62));
+  if (w < 2) return fx;
+  auto limbs = [](int64_t b, int32_t (&to)[2]) {
+    to[0] = int32_t(b >> 31);
+    to[1] = int32_t(b & 0x7fffffff);
+  };
+  limbs((int64_t(1) << 62) - w, fx.keep);
+  limbs((w + 1) / 3, fx.w3);
+  limbs((w + 18) / 36, fx.w);
+  for (int i = 0; i < 3; ++i) {
+    const double f = std::ldexp(tforce[i], 64 - e);
+    if (!(std::fabs(f) < 0x1p56)) return fx;  // tau F below S / 256
+    fx.force[i] = std::llrint(f);
+  }
+  fx.e_in = uint32_t(1011 + e);
+  fx.e_out = uint32_t(991 + e) << 20;
+  fx.unit_in = std::ldexp(1.0, e - 64);
+  fx.unit_out = std::ldexp(1.0, e - 63);
+  fx.on = 1u;
+  return fx;
+}
+
 // Everything one sweep launch needs, passed by value.
 struct SweepArgs {
   const void* src;   // storage [19][N], post-collision state of the previous step
@@ -80,6 +123,7 @@ struct SweepArgs {
   double force[3];        // F: momentum the collision adds per step
   double tforce[3];       // tau F: the equilibrium velocity shift times rho
   float forcef[3], tforcef[3];
+  FixedArgs fx;           // FP64 lattices: the relaxation in fixed point
   // Device word a sweep sets (bit 0) when it gave up waiting for its staged loads (a
   // bounded wait ran out); the host reads and clears it at its synchronisation points.
   uint32_t* err;

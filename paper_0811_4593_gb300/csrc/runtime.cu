@@ -447,6 +447,7 @@ lbm_status lbm_create_scheme(int nx, int ny, int nz, double tau, const lbm_face_
     a.mom_coef[c][1] = float(v - double(a.mom_coef[c][0]));
   }
   const double zero[3] = {0.0, 0.0, 0.0};
+  if (prec == LBM_F64) a.fx = lbm::make_fixed(rho0, a.omega, zero);
   a.pressure = 0;
   for (int f = 0; f < 6; ++f) {
     const bool open = faces[f].kind != LBM_FACE_PERIODIC;
@@ -758,6 +759,7 @@ lbm_status lbm_set_body_force(lbm_ctx* ctx, const double force[3]) {
     a.forcef[i] = float(force[i]);
     a.tforcef[i] = float(a.tforce[i]);
   }
+  if (ctx->prec == LBM_F64) a.fx = lbm::make_fixed(ctx->rho0, a.omega, a.tforce);
   a.forced = (force[0] != 0.0 || force[1] != 0.0 || force[2] != 0.0) ? 1u : 0u;
   return LBM_OK;
 }

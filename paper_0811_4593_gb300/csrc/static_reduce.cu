@@ -85,15 +85,18 @@ extern "C" LBM_API lbm_status lbm_reduce_state_static(const void* populations, i
   switch (prec) {
     case LBM_F64:
       lbm::state_reduce_kernel<double><<<blocks, lbm::SWEEP_THREADS, 0, s>>>(
-          static_cast<const double*>(populations), N, rho0, lbm::floor_neg(rho0), velocity_snapshot, partials);
+          static_cast<const double*>(populations), N, rho0, lbm::floor_neg(rho0), lbm::readout_fixed<double>(rho0),
+          velocity_snapshot, partials);
       break;
     case LBM_F32:
       lbm::state_reduce_kernel<float><<<blocks, lbm::SWEEP_THREADS, 0, s>>>(
-          static_cast<const float*>(populations), N, rho0, lbm::floor_neg(rho0), velocity_snapshot, partials);
+          static_cast<const float*>(populations), N, rho0, lbm::floor_neg(rho0), lbm::readout_fixed<float>(rho0),
+          velocity_snapshot, partials);
       break;
     default:
       lbm::state_reduce_kernel<__half><<<blocks, lbm::SWEEP_THREADS, 0, s>>>(
-          static_cast<const __half*>(populations), N, rho0, lbm::floor_neg(rho0), velocity_snapshot, partials);
+          static_cast<const __half*>(populations), N, rho0, lbm::floor_neg(rho0), lbm::readout_fixed<__half>(rho0),
+          velocity_snapshot, partials);
       break;
   }
   cudaError_t e = cudaGetLastError();
