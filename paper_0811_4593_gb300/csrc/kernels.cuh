@@ -954,6 +954,19 @@ __device__ __forceinline__ Moments<T> stored_moments(const T (&h)[Q], double rho
   return moments(h, T(ref_rho<S>(rho0)));
 }
 
+// Closure of one node: its geometry rule (word lm), or its box face, edge or corner.
+template <bool GEOM, typename T>
+__device__ __forceinline__ void close_node(const SweepArgs& a, uint32_t lm, int code, uint32_t x, uint32_t y, uint32_t z,
+                                           T (&h)[Q]) {
+  if constexpr (GEOM) {
+    const uint32_t rule = (lm >> RULE_SHIFT) & RULE_BITS;
+    if (rule != 0u) apply_rule<1, 62>(rule, h, ref_density<T>(a));
+    else if (code != 0 && !(lm & SOLID_NODE)) apply_boundary(code, a, x, y, z, h);
+  } else {
+    if (code != 0) apply_boundary(code, a, x, y, z, h);
+  }
+}
+
 // Moments, residual terms and relaxation of one node on its closed populations. FP64
 // nodes whose populations lie in the windows of fixed64.cuh are relaxed there; with
 // RESID their density and velocity are the fixed-point sums rounded to double.
@@ -1086,17 +1099,11 @@ __device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk) {
       });
     }
     const bool solid = (lm & SOLID_NODE) != 0u;
-    const uint32_t rule = (lm >> RULE_SHIFT) & RULE_BITS;
     const int fx = px ? 0 : (x == 0 ? 1 : (x == a.nx - 1 ? 2 : 0));
     const int fy = py ? 0 : (y == 0 ? 1 : (y == a.ny - 1 ? 2 : 0));
     const int fz = pz ? 0 : (z == 0 ? 1 : (z == a.nz - 1 ? 2 : 0));
     const int code = fx + 3 * fy + 9 * fz;
-    if constexpr (GEOM) {
-      if (rule != 0u) apply_rule<1, 62>(rule, h, ref_density<T>(a));
-      else if (code != 0 && !solid) apply_boundary(code, a, x, y, z, h);
-    } else {
-      if (code != 0) apply_boundary(code, a, x, y, z, h);
-    }
+    close_node<GEOM>(a, lm, code, x, y, z, h);
     relax_node<S, RESID, GEOM>(a, h, cell, solid, terms);
     static_for<0, Q>([&](auto kc) {
       constexpr int k = decltype(kc)::value;
@@ -1694,6 +1701,10 @@ __global__ void __launch_bounds__(SWEEP_THREADS)
   }
 }
 
+}  // namespace lbm
+#include "resident.cuh"
+namespace lbm {
+
 // ---------------------------------------------------------------------------------
 // Launchers.
 // ---------------------------------------------------------------------------------
@@ -1848,6 +1859,9 @@ static inline uint32_t bounds_errors_impl() {
 #define LBM_INSTANTIATE(S)                                                                              \
   template <> cudaError_t launch_sweep<S>(const SweepArgs& a, bool resid, int mode, cudaStream_t s) {   \
     return launch_sweep_impl<S>(a, resid, mode, s);                                                     \
+  }                                                                                                     \
+  template <> cudaError_t launch_resident<S>(const SweepArgs& a, int steps, bool swapped, cudaStream_t s) { \
+    return launch_resident_impl<S>(a, steps, swapped, s);                                               \
   }                                                                                                     \
   template <> cudaError_t launch_init<S>(void* dst, uint32_t N, double rho0, cudaStream_t s) {          \
     return launch_init_impl<S>(dst, N, rho0, s);                                                        \

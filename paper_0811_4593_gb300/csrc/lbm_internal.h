@@ -182,8 +182,18 @@ __host__ __device__ inline uint32_t fold_groups(uint32_t nblocks) { return (nblo
 // rows of a partial-sum buffer: the sweep's blocks, then the fold's groups
 inline uint32_t partial_rows(uint32_t nblocks) { return nblocks + fold_groups(nblocks); }
 
+// The multi-step kernel of small lattices (resident.cuh): nodes a CTA holds at most, the
+// largest (non-portable) cluster, and the shortest run of steps it is taken for (below,
+// loading and storing the state costs as much as the launches).
+constexpr uint32_t RESIDENT_THREADS = 512;
+constexpr uint32_t RESIDENT_CTAS = 16;
+constexpr uint32_t RESIDENT_NODES = RESIDENT_THREADS * RESIDENT_CTAS;
+constexpr int RESIDENT_MIN_STEPS = 16;
+
 // mode: 0 A/B pull, 1 AA gather-scatter step, 2 AA in-place step (see kernels.cuh)
 template <typename S> cudaError_t launch_sweep(const SweepArgs& a, bool resid, int mode, cudaStream_t s);
+// `steps` steps of a small lattice in one launch (resident.cuh), from src to dst
+template <typename S> cudaError_t launch_resident(const SweepArgs& a, int steps, bool swapped, cudaStream_t s);
 template <typename S> cudaError_t launch_init(void* dst, uint32_t N, double rho0, cudaStream_t s);
 // swapped: the state holds f_k in slot -k (an AA lattice between step pairs)
 template <typename S> cudaError_t launch_macros(const void* src, uint32_t N, double rho0, void* rho,

@@ -278,6 +278,47 @@ cudaError_t dispatch_sweep(lbm_ctx* ctx, bool resid) {
   }
 }
 
+cudaError_t dispatch_resident(lbm_ctx* ctx, int n) {
+  const bool swapped = ctx->scheme == LBM_SCHEME_AA;
+  switch (ctx->prec) {
+    case LBM_F64: return lbm::launch_resident<double>(ctx->args, n, swapped, ctx->stream);
+    case LBM_F32: return lbm::launch_resident<float>(ctx->args, n, swapped, ctx->stream);
+    default: return lbm::launch_resident<__half>(ctx->args, n, swapped, ctx->stream);
+  }
+}
+
+// Issues n plain steps: one launch each, or for a small lattice all of them (an even
+// number for AA, whose state it reads and leaves between step pairs) in one.
+lbm_status issue_steps(lbm_ctx* ctx, int n) {
+  const bool aa = ctx->scheme == LBM_SCHEME_AA;
+  const int m = aa ? n & ~1 : n;
+  if (ctx->N <= lbm::RESIDENT_NODES && m >= lbm::RESIDENT_MIN_STEPS && !(aa && ctx->steps % 2 != 0)) {
+    // m steps leave the state where m launches would: in the other array when m is odd
+    set_direction(ctx, ctx->cur);
+    if (m % 2 == 0) {
+      ctx->args.dst = ctx->buf[ctx->cur];
+      for (int k = 0; k < 19; ++k) ctx->args.dst_pop[k] = const_cast<void*>(ctx->args.src_pop[k]);
+    }
+    const cudaError_t e = dispatch_resident(ctx, m);
+    if (e == cudaSuccess) {
+      if (!aa) ctx->cur ^= m & 1;
+      ctx->steps += m;
+      ctx->launches += 1;
+      n -= m;
+    } else if (e != cudaErrorNotSupported) {
+      return cuda_fail(ctx, e, "multi-step launch");
+    }
+  }
+  for (int i = 0; i < n; ++i) {
+    set_direction(ctx, ctx->cur);
+    LBM_CUDA(ctx, dispatch_sweep(ctx, false), "sweep launch");
+    if (!aa) ctx->cur ^= 1;
+    ctx->steps += 1;
+    ctx->launches += 1;
+  }
+  return LBM_OK;
+}
+
 // Observations (macros, residual, population copies) need the post-collision state:
 // always for A/B, between step pairs for AA (where population k sits in slot -k).
 lbm_status require_observable(lbm_ctx* ctx) {
@@ -506,14 +547,7 @@ lbm_status lbm_step(lbm_ctx* ctx, int n) {
   DeviceGuard g(ctx->device);
   if (!g.ok) return fail(ctx, LBM_ERR_CUDA, "cannot make device %d current", ctx->device);
   if (lbm_status st0 = settle(ctx); st0 != LBM_OK) return st0;
-  for (int i = 0; i < n; ++i) {
-    set_direction(ctx, ctx->cur);
-    LBM_CUDA(ctx, dispatch_sweep(ctx, false), "sweep launch");
-    if (ctx->scheme == LBM_SCHEME_AB) ctx->cur ^= 1;
-    ctx->steps += 1;
-    ctx->launches += 1;
-  }
-  return LBM_OK;
+  return issue_steps(ctx, n);
 }
 
 lbm_status lbm_step_residual(lbm_ctx* ctx, int n, double* residual, double* mass) {
@@ -527,14 +561,7 @@ lbm_status lbm_step_residual(lbm_ctx* ctx, int n, double* residual, double* mass
   if (lbm_status st0 = require_observable(ctx); st0 != LBM_OK) return st0;
   lbm_status st = ensure_reduction_buffers(ctx);
   if (st != LBM_OK) return st;
-  // the n - 1 plain steps (an odd count for AA: issue them one by one)
-  for (int i = 0; i < n - 1; ++i) {
-    set_direction(ctx, ctx->cur);
-    LBM_CUDA(ctx, dispatch_sweep(ctx, false), "sweep launch");
-    if (ctx->scheme == LBM_SCHEME_AB) ctx->cur ^= 1;
-    ctx->steps += 1;
-    ctx->launches += 1;
-  }
+  if (st = issue_steps(ctx, n - 1); st != LBM_OK) return st;
   set_direction(ctx, ctx->cur);
   LBM_CUDA(ctx, dispatch_sweep(ctx, true), "residual sweep launch");
   if (ctx->scheme == LBM_SCHEME_AB) ctx->cur ^= 1;
