@@ -204,24 +204,39 @@ __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float t) {
   lo = __fadd_rn(lo, e);
 }
 
-// Velocity of a face node in the compute type, and 1 / (1 - u.n) in double.
+// A number of the density relations: double in FP64 sweeps, a float pair (about 47 bits)
+// in float ones. The FP64 pipe issues a warp instruction in about 19 SM cycles, so the
+// six conversions and operations that formed a float node's density in double took half
+// of a face node's time in short-row and small lattices; rounded to float, the pair's
+// result differs from the double one in about one of 2^21 cases, by one ulp.
+template <typename T> struct WideOf { using type = double; };
+template <> struct WideOf<float> { using type = fpair; };
+template <typename T> using Wide = typename WideOf<T>::type;
+
+// Prescribed values of a face node. Velocity face: u and wide(1 / (1 - u.n)). Pressure
+// face: the tangential velocity, wide(1 / rho_p) (FP64: rho_p itself), and rho_p and
+// rho_p - ref in the compute type.
 template <typename T>
 struct FaceVals {
   T u[3];
-  double inv;
+  Wide<T> inv;
+  T rho, drho;
 };
+
+// The reference density of the register values, wide.
+template <typename T> __device__ __forceinline__ Wide<T> ref_density(const SweepArgs& a);
+template <> __device__ __forceinline__ double ref_density<double>(const SweepArgs&) { return 0.0; }
+template <> __device__ __forceinline__ fpair ref_density<float>(const SweepArgs& a) { return {a.rho0f, a.rho0_lo}; }
 
 // The relation's sum over the shifted populations of a plane with inward normal
 // SG * e_A: in-plane populations once, outgoing ones twice (its weights sum to 1, so
 // the plane's density relation reads rho (1 - u.n) = ref + S). FP64: accumulated in
 // double. Float sweeps: accumulated as a float pair hi + lo with TwoSum, which is
 // exact except for the float rounding of lo's own sum of the 14 error terms; that
-// leaves an error below about 14^2 2^-48 (~7e-13) of the largest partial sum, against
-// 14 2^-53 (~2e-15) for accumulation in double -- both far below the float rounding of
-// the populations, and the pair costs no FP64 work on the face nodes until the final
-// conversion.
+// leaves an error below about 14^2 2^-48 (~7e-13) of the largest partial sum, far below
+// the float rounding of the populations.
 template <int A, int SG, typename T>
-__device__ __forceinline__ double relation_sum(const T (&h)[Q]) {
+__device__ __forceinline__ Wide<T> relation_sum(const T (&h)[Q]) {
   if constexpr (std::is_same<T, double>::value) {
     double S = 0.0;
     static_for<0, Q>([&](auto kc) {
@@ -239,8 +254,28 @@ __device__ __forceinline__ double relation_sum(const T (&h)[Q]) {
       if constexpr (cn == 0) two_sum_acc(hi, lo, h[k]);
       else if constexpr (cn < 0) two_sum_acc(hi, lo, __fmul_rn(2.0f, h[k]));
     });
-    return double(hi) + double(lo);
+    return {hi, lo};
   }
+}
+
+// (ref + S) inv in the compute type, and as hi + lo for float
+__device__ __forceinline__ fpair times(fpair ref, fpair S, fpair inv) {
+  const fpair a = sum_of(ref, S);
+  const float p = __fmul_rn(a.hi, inv.hi);
+  const float e = __fmaf_rn(a.hi, inv.lo, __fmaf_rn(a.lo, inv.hi, __fmaf_rn(a.hi, inv.hi, -p)));
+  return {p, e};
+}
+__device__ __forceinline__ double relation_density(double ref, double S, double inv) { return (ref + S) * inv; }
+__device__ __forceinline__ float relation_density(fpair ref, fpair S, fpair inv) {
+  const fpair r = times(ref, S, inv);
+  return __fadd_rn(r.hi, r.lo);
+}
+// u.n = 1 - (ref + S) / rho_p
+__device__ __forceinline__ double relation_velocity(double ref, double S, double rho_p) { return 1.0 - (ref + S) / rho_p; }
+__device__ __forceinline__ float relation_velocity(fpair ref, fpair S, fpair inv) {
+  const fpair r = times(ref, S, inv);
+  const fpair v = sum_of(fpair{1.0f, 0.0f}, fpair{-r.hi, -r.lo});
+  return __fadd_rn(v.hi, v.lo);
 }
 
 // Unknown populations of a plane with inward normal SG * e_A, given the node's density
@@ -287,24 +322,23 @@ __device__ __forceinline__ void fill_unknowns(T (&h)[Q], T rho, const T (&u)[3])
 }
 
 // On-site velocity closure (eq. uin and the appendix relations): the density
-// rho = (ref + S) / (1 - u.n), formed in double (fv.inv = 1 / (1 - u.n) from the host),
+// rho = (ref + S) / (1 - u.n), formed wide (fv.inv = 1 / (1 - u.n) from the host),
 // then the unknown populations.
 template <int A, int SG, typename T>
-__device__ __forceinline__ void close_face(T (&h)[Q], const FaceVals<T>& fv, double ref) {
-  const T rho = T((ref + relation_sum<A, SG>(h)) * fv.inv);
+__device__ __forceinline__ void close_face(T (&h)[Q], const FaceVals<T>& fv, Wide<T> ref) {
+  const T rho = relation_density(ref, relation_sum<A, SG>(h), fv.inv);
   fill_unknowns<A, SG>(h, rho, fv.u);
 }
 
-// Pressure variant (eq. rhoin and the appendix relations): the density rho_p
-// (fv.inv) and the tangential velocity are prescribed; the normal velocity
-// u.n = 1 - (ref + S) / rho_p, formed in double; then the unknown populations.
+// Pressure variant (eq. rhoin and the appendix relations): the density rho_p and the
+// tangential velocity are prescribed; the normal velocity u.n = 1 - (ref + S) / rho_p,
+// formed wide; then the unknown populations.
 template <int A, int SG, typename T>
-__device__ __forceinline__ void close_face_pressure(T (&h)[Q], const FaceVals<T>& fv, double ref) {
-  const double rho_p = fv.inv;
-  const double un = 1.0 - (ref + relation_sum<A, SG>(h)) / rho_p;
+__device__ __forceinline__ void close_face_pressure(T (&h)[Q], const FaceVals<T>& fv, Wide<T> ref) {
+  const T un = relation_velocity(ref, relation_sum<A, SG>(h), fv.inv);
   T u[3] = {fv.u[0], fv.u[1], fv.u[2]};
-  u[A] = T(double(SG) * un);
-  fill_unknowns<A, SG>(h, T(rho_p), u);
+  u[A] = sgn<SG>(un);
+  fill_unknowns<A, SG>(h, fv.rho, u);
 }
 
 // Concave no-slip edge of the planes with inward normals n1 = S1 e_A1 and
@@ -395,11 +429,10 @@ __device__ __forceinline__ void close_corner(T (&h)[Q], bool pressure, T drho_p)
   h[Q - 1] = T(12) * fb;
 }
 
-// Prescribed velocity of face (A, SG) at node (x, y, z): from the face's node table
-// when it has one, else the face's uniform value.
-template <int A, int SG, typename T>
-__device__ __forceinline__ FaceVals<T> face_values(const SweepArgs& a, uint32_t x, uint32_t y, uint32_t z) {
-  constexpr int f = 2 * A + (SG > 0 ? 0 : 1);
+// Prescribed values of face f (on axis A) at node (x, y, z): from the face's node table
+// when it has one, else the face's uniform ones.
+template <int A, typename T>
+__device__ __forceinline__ FaceVals<T> face_values(const SweepArgs& a, int f, uint32_t x, uint32_t y, uint32_t z) {
   const FaceBC& fb = a.face[f];
   FaceVals<T> v;
   if (fb.tab) {
@@ -414,33 +447,18 @@ __device__ __forceinline__ FaceVals<T> face_values(const SweepArgs& a, uint32_t 
       v.u[0] = a0.x;
       v.u[1] = a0.y;
       v.u[2] = a1.x;
-      v.inv = a1.y;
+      v.inv = v.rho = v.drho = a1.y;
     } else {
       const float4 b = __ldg(reinterpret_cast<const float4*>(p) + 2);
-      v.u[0] = b.x;
-      v.u[1] = b.y;
-      v.u[2] = b.z;
-      v.inv = __ldg(&p->inv);
+      const float4 c = __ldg(reinterpret_cast<const float4*>(p) + 3);
+      v = {{b.x, b.y, b.z}, {b.w, c.x}, c.y, c.z};
     }
   } else {
-    if constexpr (std::is_same<T, double>::value) {
-      v.u[0] = fb.uni.u[0];
-      v.u[1] = fb.uni.u[1];
-      v.u[2] = fb.uni.u[2];
-    } else {
-      v.u[0] = fb.uni.uf[0];
-      v.u[1] = fb.uni.uf[1];
-      v.u[2] = fb.uni.uf[2];
-    }
-    v.inv = fb.uni.inv;
+    const FaceNode& n = fb.uni;
+    if constexpr (std::is_same<T, double>::value) v = {{n.u[0], n.u[1], n.u[2]}, n.inv, n.inv, n.inv};
+    else v = {{n.uf[0], n.uf[1], n.uf[2]}, {n.inv_hi, n.inv_lo}, n.rho, n.drho};
   }
   return v;
-}
-
-// Reference density of the register values: 0 for FP64 (unshifted), rho0 otherwise.
-template <typename T>
-__device__ __forceinline__ double ref_density(const SweepArgs& a) {
-  return std::is_same<T, double>::value ? 0.0 : a.rho0;
 }
 
 template <int A, int SG>
@@ -448,9 +466,42 @@ constexpr int face_id() { return 2 * A + (SG > 0 ? 0 : 1); }
 
 template <int A, int SG, typename T>
 __device__ __forceinline__ void face_case(const SweepArgs& a, uint32_t x, uint32_t y, uint32_t z, T (&h)[Q]) {
-  const FaceVals<T> fv = face_values<A, SG, T>(a, x, y, z);
+  const FaceVals<T> fv = face_values<A, T>(a, face_id<A, SG>(), x, y, z);
   if (a.pressure & (1u << face_id<A, SG>())) close_face_pressure<A, SG>(h, fv, ref_density<T>(a));
   else close_face<A, SG>(h, fv, ref_density<T>(a));
+}
+
+// Population k with c_x reversed.
+__host__ __device__ constexpr int mirror_x(int k) { return vel_index(-cx(k), cy(k), cz(k)); }
+
+// Both x faces in one body: a node of the high face is mirrored in x, closed as one of
+// the low face and mirrored back. Warps of short rows hold nodes of both faces and would
+// run the body twice. The mirrored sums take their terms in the same order, so the bits
+// are those of the face's own body.
+template <typename T>
+__device__ __forceinline__ void x_face_case(const SweepArgs& a, bool high, uint32_t x, uint32_t y, uint32_t z, T (&h)[Q]) {
+  auto mirror = [&] {
+    static_for<0, Q>([&](auto kc) {
+      constexpr int k = decltype(kc)::value, m = mirror_x(k);
+      if constexpr (cx(k) > 0) {
+        const T t = high ? h[m] : h[k];
+        h[m] = high ? h[k] : h[m];
+        h[k] = t;
+      }
+    });
+  };
+  FaceVals<T> fv = face_values<0, T>(a, high ? 1 : 0, x, y, z);
+  fv.u[0] = high ? -fv.u[0] : fv.u[0];
+  mirror();
+  if (a.pressure & (high ? 2u : 1u)) close_face_pressure<0, +1>(h, fv, ref_density<T>(a));
+  else close_face<0, +1>(h, fv, ref_density<T>(a));
+  mirror();
+}
+
+// rho_p - ref of a pressure face next to an edge or corner
+template <int A, int SG, typename T>
+__device__ __forceinline__ T face_drho(const SweepArgs& a, uint32_t x, uint32_t y, uint32_t z) {
+  return face_values<A, T>(a, face_id<A, SG>(), x, y, z).drho;
 }
 
 // Edge of faces (A1, S1) and (A2, S2); when one of them is a pressure face its density
@@ -459,8 +510,7 @@ template <int A1, int S1, int A2, int S2, typename T>
 __device__ __forceinline__ void edge_case(const SweepArgs& a, uint32_t x, uint32_t y, uint32_t z, T (&h)[Q]) {
   constexpr uint32_t b1 = 1u << face_id<A1, S1>(), b2 = 1u << face_id<A2, S2>();
   if (a.pressure & (b1 | b2)) {
-    const double rp = (a.pressure & b1) ? face_values<A1, S1, T>(a, x, y, z).inv : face_values<A2, S2, T>(a, x, y, z).inv;
-    close_edge<A1, S1, A2, S2>(h, true, T(rp - ref_density<T>(a)));
+    close_edge<A1, S1, A2, S2>(h, true, (a.pressure & b1) ? face_drho<A1, S1, T>(a, x, y, z) : face_drho<A2, S2, T>(a, x, y, z));
   } else {
     close_edge<A1, S1, A2, S2>(h, false, T(0));
   }
@@ -470,10 +520,9 @@ template <int SX, int SY, int SZ, typename T>
 __device__ __forceinline__ void corner_case(const SweepArgs& a, uint32_t x, uint32_t y, uint32_t z, T (&h)[Q]) {
   constexpr uint32_t bx = 1u << face_id<0, SX>(), by = 1u << face_id<1, SY>(), bz = 1u << face_id<2, SZ>();
   if (a.pressure & (bx | by | bz)) {
-    const double rp = (a.pressure & bx)   ? face_values<0, SX, T>(a, x, y, z).inv
-                      : (a.pressure & by) ? face_values<1, SY, T>(a, x, y, z).inv
-                                          : face_values<2, SZ, T>(a, x, y, z).inv;
-    close_corner<SX, SY, SZ>(h, true, T(rp - ref_density<T>(a)));
+    close_corner<SX, SY, SZ>(h, true, (a.pressure & bx)   ? face_drho<0, SX, T>(a, x, y, z)
+                                      : (a.pressure & by) ? face_drho<1, SY, T>(a, x, y, z)
+                                                          : face_drho<2, SZ, T>(a, x, y, z));
   } else {
     close_corner<SX, SY, SZ>(h, false, T(0));
   }
@@ -485,8 +534,8 @@ __device__ __forceinline__ void apply_boundary(int code, const SweepArgs& a, uin
                                                uint32_t z, T (&h)[Q]) {
   switch (code) {
     // faces
-    case 1: face_case<0, +1>(a, x, y, z, h); break;
-    case 2: face_case<0, -1>(a, x, y, z, h); break;
+    case 1:
+    case 2: x_face_case(a, code == 2, x, y, z, h); break;
     case 3: face_case<1, +1>(a, x, y, z, h); break;
     case 6: face_case<1, -1>(a, x, y, z, h); break;
     case 9: face_case<2, +1>(a, x, y, z, h); break;
@@ -579,10 +628,12 @@ __device__ __forceinline__ void close_junction(T (&h)[Q]) {
 // edges with bulk normal c_R, 19..26 corners, 27..50 junctions, 51..62 convex edges
 // with bulk normal c_(R-44).
 template <int R, typename T>
-__device__ __forceinline__ void rule_case(T (&h)[Q], double ref) {
+__device__ __forceinline__ void rule_case(T (&h)[Q], Wide<T> ref) {
   if constexpr (R >= 1 && R <= 6) {
     constexpr int k = R - 1;
-    const FaceVals<T> rest = {{T(0), T(0), T(0)}, 1.0};
+    FaceVals<T> rest = {};
+    if constexpr (std::is_same<T, double>::value) rest.inv = 1.0;
+    else rest.inv.hi = 1.0f;
     close_face<axis_of(k), sign_of(k)>(h, rest, ref);
   } else if constexpr (R >= 7 && R <= 18) {
     constexpr int k = R - 1;
@@ -605,7 +656,7 @@ __device__ __forceinline__ void rule_case(T (&h)[Q], double ref) {
 }
 
 template <int LO, int HI, typename T>
-__device__ __forceinline__ void apply_rule(uint32_t r, T (&h)[Q], double ref) {
+__device__ __forceinline__ void apply_rule(uint32_t r, T (&h)[Q], Wide<T> ref) {
   if constexpr (LO == HI) {
     rule_case<LO>(h, ref);
   } else {

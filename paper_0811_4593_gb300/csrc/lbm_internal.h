@@ -39,14 +39,18 @@ inline float floor_neg(double rho0) {
   return double(f) > -rho0 ? std::nextafter(f, -INFINITY) : f;
 }
 
-// One boundary-face node as the sweep reads it. Velocity face: the prescribed velocity
-// in double and float, and 1 / (1 - u.n) for the density relation (n = inward normal),
-// formed in double on the host. Pressure face: the tangential velocity (normal part
-// zero) in double and float, and the prescribed density in `inv`.
+// One boundary-face node as the sweep reads it, the first half by FP64 sweeps, the second
+// by float ones. Velocity face: the prescribed velocity and 1 / (1 - u.n) for the density
+// relation (n = inward normal), formed in double on the host, for float sweeps as a pair
+// hi + lo. Pressure face: the tangential velocity (normal part zero), the prescribed
+// density in `inv`, and for float sweeps its reciprocal as a pair, the density and its
+// difference from rho0.
 struct __align__(16) FaceNode {
   double u[3];
   double inv;
   float uf[3];
+  float inv_hi, inv_lo;
+  float rho, drho;
   float pad;
 };
 
@@ -113,6 +117,7 @@ struct SweepArgs {
   double rho0;
   double omega;       // 1 / tau
   float rho0f, omegaf;
+  float rho0_lo;      // rho0 - rho0f
   float neg_rho0;     // floor_neg(rho0)
   float mom_coef[2][2];  // omegaf / 6 and omegaf / 12 as hi + lo float pairs
   FaceBC face[6];

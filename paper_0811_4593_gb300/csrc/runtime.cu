@@ -179,16 +179,20 @@ void ctx_free_all(lbm_ctx* ctx) {
   ctx->device_bytes = 0;
 }
 
-// Sweep record of one node of face f. Velocity face: u in double and float and
-// 1 / (1 - u.n) in double (n the inward normal; |u.n| < 1 is validated). Pressure
-// face: the tangential part of u and, in the `inv` field, the prescribed density.
-lbm::FaceNode face_node(int f, const double* u, bool pressure, double rho) {
+// Sweep record of one node of face f. Velocity face: u and 1 / (1 - u.n) (n the inward
+// normal; |u.n| < 1 is validated). Pressure face: the tangential part of u and the
+// prescribed density (see FaceNode).
+lbm::FaceNode face_node(int f, const double* u, bool pressure, double rho, double rho0) {
   lbm::FaceNode n{};
   for (int j = 0; j < 3; ++j) n.u[j] = (pressure && j == f / 2) ? 0.0 : u[j];
   for (int j = 0; j < 3; ++j) n.uf[j] = float(n.u[j]);
   const double un = (f % 2 == 0 ? 1.0 : -1.0) * u[f / 2];
-  n.inv = pressure ? rho : 1.0 / (1.0 - un);
-  n.pad = 0.0f;
+  const double inv = pressure ? 1.0 / rho : 1.0 / (1.0 - un);
+  n.inv = pressure ? rho : inv;
+  n.inv_hi = float(inv);
+  n.inv_lo = float(inv - double(n.inv_hi));
+  n.rho = float(rho);
+  n.drho = float(rho - rho0);
   return n;
 }
 
@@ -477,6 +481,7 @@ lbm_status lbm_create_scheme(int nx, int ny, int nz, double tau, const lbm_face_
   a.rho0 = rho0;
   a.omega = 1.0 / tau;
   a.rho0f = float(rho0);
+  a.rho0_lo = float(rho0 - double(a.rho0f));
   a.neg_rho0 = lbm::floor_neg(rho0);
   a.omegaf = float(1.0 / tau);
   // 3 omega w_i of the BGK update's momentum term for the float sweep, as hi + lo
@@ -495,7 +500,7 @@ lbm_status lbm_create_scheme(int nx, int ny, int nz, double tau, const lbm_face_
     const bool pres = faces[f].kind == LBM_FACE_PRESSURE;
     if (pres) a.pressure |= 1u << f;
     a.face[f].tab = nullptr;
-    a.face[f].uni = face_node(f, open ? faces[f].u : zero, pres, pres ? faces[f].rho : 0.0);
+    a.face[f].uni = face_node(f, open ? faces[f].u : zero, pres, pres ? faces[f].rho : 0.0, rho0);
     const bool per_node = open && (faces[f].u_table || (pres && faces[f].rho_table));
     if (per_node) {
       const size_t m = size_t(face_n1(f, nx, ny)) * face_n2(f, ny, nz);
@@ -503,7 +508,7 @@ lbm_status lbm_create_scheme(int nx, int ny, int nz, double tau, const lbm_face_
       for (size_t i = 0; i < m; ++i) {
         const double* u = faces[f].u_table ? faces[f].u_table + 3 * i : faces[f].u;
         const double r = pres ? (faces[f].rho_table ? faces[f].rho_table[i] : faces[f].rho) : 0.0;
-        host[i] = face_node(f, u, pres, r);
+        host[i] = face_node(f, u, pres, r, rho0);
       }
       const size_t bytes = m * sizeof(lbm::FaceNode);
       void* t = ctx_alloc(ctx, bytes);

@@ -30,7 +30,7 @@ def footprint_bytes(nx: int, ny: int, nz: int, precision: str, scheme: str = "ab
     reduction scalars."""
     n = nx * ny * nz
     blocks = (n + 255) // 256
-    faces = 2 * (ny * nz + nx * nz + nx * ny) * 48
+    faces = 2 * (ny * nz + nx * nz + nx * ny) * 64
     buffers = 1 if scheme == "aa" else 2
     return buffers * 19 * STORAGE_BYTES[precision] * n + 3 * COMPUTE_BYTES[precision] * n + 32 * blocks + faces + 32
 
