@@ -108,6 +108,17 @@ __device__ __forceinline__ uint32_t chk(uint32_t i, uint32_t limit) {
 __device__ __forceinline__ uint32_t chk(uint32_t i, uint32_t) { return i; }
 #endif
 
+// Programmatic dependent launch: consecutive sweeps of a stream are launched with the
+// serialisation relaxed (launch_after), so the next sweep's blocks are placed while the
+// last ones of this sweep run, and wait here, before their first access to memory, until
+// it has completed and its stores are visible. `index` ties every address to the wait:
+// loads written as plain functions of a pointer may otherwise be moved above it. Without
+// such a launch both instructions do nothing.
+__device__ __forceinline__ void wait_for_previous_sweep(uint32_t& index) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" : "+r"(index)::"memory");
+}
+
 // Signed sums whose first term is taken as it is (negation is exact), so that no
 // rounded addition of zero is ever issued.
 template <int SGN, typename T>
@@ -1201,7 +1212,9 @@ struct SweepOccupancy<double, RESID, BATCHED, MODE, GEOM> {
 template <typename S, bool RESID, int MODE, bool GEOM>
 __global__ void __launch_bounds__(SWEEP_THREADS, (SweepOccupancy<S, RESID, false, MODE, GEOM>::blocks))
     sweep_kernel(const __grid_constant__ SweepArgs a) {
-  sweep_block<S, RESID, MODE, GEOM>(a, blockIdx.x);
+  uint32_t blk = blockIdx.x;
+  wait_for_previous_sweep(blk);
+  sweep_block<S, RESID, MODE, GEOM>(a, blk);
 }
 
 // ---------------------------------------------------------------------------------
@@ -1276,7 +1289,8 @@ __device__ __forceinline__ void close_lane(int code, const SweepArgs& a, uint32_
 template <typename S, int MODE>
 __global__ void __launch_bounds__(SWEEP_THREADS, 4) sweep_pair_kernel(const __grid_constant__ SweepArgs a) {
   static_assert(std::is_same<S, __half>::value, "the paired sweep is for binary16 storage");
-  const uint32_t pair = blockIdx.x * SWEEP_THREADS + threadIdx.x;
+  uint32_t pair = blockIdx.x * SWEEP_THREADS + threadIdx.x;
+  wait_for_previous_sweep(pair);
   if (pair >= (a.N >> 1)) return;
   const uint32_t q1 = fdiv(a.div_nxh, pair);
   const uint32_t x0 = 2u * (pair - q1 * (a.nx >> 1));
@@ -1483,6 +1497,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 3) sweep_rows_kernel(const __gri
   extern __shared__ __align__(128) unsigned char rows_smem[];
   __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES];
   const uint32_t nx = a.nx, nrows = a.ny * a.nz;
+  uint32_t first_group = blockIdx.x;
   const bool px = a.periodic & 1u, py = a.periodic & 2u, pz = a.periodic & 4u;
   const __half* stage0 = reinterpret_cast<const __half*>(rows_smem);
   if (threadIdx.x == 0) {
@@ -1495,6 +1510,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 3) sweep_rows_kernel(const __gri
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   __syncthreads();
+  wait_for_previous_sweep(first_group);
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
   // a stage holds R consecutive rows, R * nx / 2 >= the consumer threads when nx allows
   const uint32_t R = (ROWS_STAGE_NODES + nx - 1) / nx;
@@ -1507,7 +1523,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 3) sweep_rows_kernel(const __gri
     const uint32_t row_bytes = nx * uint32_t(sizeof(__half));
     uint32_t i = 0;
     for (;; ++i) {
-      const uint32_t g = blockIdx.x + i * gridDim.x;
+      const uint32_t g = first_group + i * gridDim.x;
       if (g >= ngroups) break;
       const int s = int(i % STAGES);
       if (i >= uint32_t(STAGES) &&
@@ -1542,7 +1558,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 3) sweep_rows_kernel(const __gri
     }
     // the copies of the last (up to STAGES) groups issued may still be in flight: the
     // consumers wait for them; if the loop ended early, wait for them here (bounded)
-    if (blockIdx.x + i * gridDim.x < ngroups) {
+    if (first_group + i * gridDim.x < ngroups) {
       for (uint32_t j = (i > uint32_t(STAGES) ? i - STAGES : 0); j < i; ++j)
         (void)mbar_wait_bounded(smem_u32(&full[j % STAGES]), (j / STAGES) & 1u, STAGE_WAIT_LIMIT_NS);
     }
@@ -1551,7 +1567,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 3) sweep_rows_kernel(const __gri
   // consumers: 256 threads over the node pairs of the group's rows
   const uint32_t npairs = nx >> 1;
   for (uint32_t i = 0;; ++i) {
-    const uint32_t g = blockIdx.x + i * gridDim.x;
+    const uint32_t g = first_group + i * gridDim.x;
     if (g >= ngroups) break;
     const int s = int(i % STAGES);
     if (!mbar_wait_bounded(smem_u32(&full[s]), (i / STAGES) & 1u, STAGE_WAIT_LIMIT_NS)) {
@@ -1759,11 +1775,28 @@ namespace lbm {
 // ---------------------------------------------------------------------------------
 // Launchers.
 // ---------------------------------------------------------------------------------
+// Launches a sweep that may start before the previous kernel of the stream has ended; it
+// waits for it itself (wait_for_previous_sweep). Measured per step: 32^3 FP32 with a body
+// force 6.3 -> 5.6 us, 256 x 64 x 64 FP32 27.4 -> 24.6 us.
+inline cudaError_t launch_after(void (*kernel)(SweepArgs), uint32_t grid, uint32_t threads, size_t smem,
+                                const SweepArgs& a, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
 template <typename S, int MODE, bool GEOM>
-void launch_sweep_mode(const SweepArgs& a, bool resid, cudaStream_t s) {
-  const uint32_t blocks = sweep_blocks(a.N);
-  if (resid) sweep_kernel<S, true, MODE, GEOM><<<blocks, SWEEP_THREADS, 0, s>>>(a);
-  else sweep_kernel<S, false, MODE, GEOM><<<blocks, SWEEP_THREADS, 0, s>>>(a);
+cudaError_t launch_sweep_mode(const SweepArgs& a, bool resid, cudaStream_t s) {
+  auto kernel = resid ? sweep_kernel<S, true, MODE, GEOM> : sweep_kernel<S, false, MODE, GEOM>;
+  return launch_after(kernel, sweep_blocks(a.N), SWEEP_THREADS, 0, a, s);
 }
 
 // Stages of the row-staged sweep's shared-memory ring.
@@ -1779,8 +1812,7 @@ cudaError_t launch_rows(const SweepArgs& a, cudaStream_t s) {
   const uint32_t R = (ROWS_STAGE_NODES + a.nx - 1) / a.nx;  // rows per stage (as the kernel)
   const size_t smem = size_t(ROWS_STAGES) * Q * R * a.nx * sizeof(__half);
   const bool fixed = R * a.nx == ROWS_STAGE_NODES;
-  const void* fn = fixed ? reinterpret_cast<const void*>(sweep_rows_kernel<ROWS_STAGES, MODE, true>)
-                         : reinterpret_cast<const void*>(sweep_rows_kernel<ROWS_STAGES, MODE, false>);
+  auto fn = fixed ? sweep_rows_kernel<ROWS_STAGES, MODE, true> : sweep_rows_kernel<ROWS_STAGES, MODE, false>;
   int dev = 0, sms = 0, per = 0, optin = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1793,9 +1825,7 @@ cudaError_t launch_rows(const SweepArgs& a, cudaStream_t s) {
   if (per < 1) return cudaErrorNotSupported;
   const uint32_t ngroups = (a.ny * a.nz + R - 1) / R;
   const uint32_t grid = uint32_t(sms * per) < ngroups ? uint32_t(sms * per) : ngroups;
-  if (fixed) sweep_rows_kernel<ROWS_STAGES, MODE, true><<<grid, ROWS_THREADS, smem, s>>>(a);
-  else sweep_rows_kernel<ROWS_STAGES, MODE, false><<<grid, ROWS_THREADS, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_after(fn, grid, ROWS_THREADS, smem, a, s);
 }
 
 template <typename S>
@@ -1808,18 +1838,16 @@ cudaError_t launch_sweep_impl(const SweepArgs& a, bool resid, int mode, cudaStre
       if (e != cudaErrorNotSupported) return e;
     }
     if (!resid && !a.links && !a.forced && (a.nx & 1u) == 0) {
-      const uint32_t blocks = sweep_blocks(a.N >> 1);
-      if (mode == STREAM_AA_GATHER) sweep_pair_kernel<S, STREAM_AA_GATHER><<<blocks, SWEEP_THREADS, 0, s>>>(a);
-      else if (mode == STREAM_AA_LOCAL) sweep_pair_kernel<S, STREAM_AA_LOCAL><<<blocks, SWEEP_THREADS, 0, s>>>(a);
-      else sweep_pair_kernel<S, STREAM_AB><<<blocks, SWEEP_THREADS, 0, s>>>(a);
-      return cudaGetLastError();
+      auto kernel = mode == STREAM_AA_GATHER  ? sweep_pair_kernel<S, STREAM_AA_GATHER>
+                    : mode == STREAM_AA_LOCAL ? sweep_pair_kernel<S, STREAM_AA_LOCAL>
+                                              : sweep_pair_kernel<S, STREAM_AB>;
+      return launch_after(kernel, sweep_blocks(a.N >> 1), SWEEP_THREADS, 0, a, s);
     }
   }
-  if (mode == STREAM_AA_GATHER) launch_sweep_mode<S, STREAM_AA_GATHER, false>(a, resid, s);
-  else if (mode == STREAM_AA_LOCAL) launch_sweep_mode<S, STREAM_AA_LOCAL, false>(a, resid, s);
-  else if (a.links || a.forced) launch_sweep_mode<S, STREAM_AB, true>(a, resid, s);
-  else launch_sweep_mode<S, STREAM_AB, false>(a, resid, s);
-  return cudaGetLastError();
+  if (mode == STREAM_AA_GATHER) return launch_sweep_mode<S, STREAM_AA_GATHER, false>(a, resid, s);
+  if (mode == STREAM_AA_LOCAL) return launch_sweep_mode<S, STREAM_AA_LOCAL, false>(a, resid, s);
+  if (a.links || a.forced) return launch_sweep_mode<S, STREAM_AB, true>(a, resid, s);
+  return launch_sweep_mode<S, STREAM_AB, false>(a, resid, s);
 }
 
 template <typename S>
