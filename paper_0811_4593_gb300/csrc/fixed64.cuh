@@ -62,8 +62,8 @@ __host__ __device__ __forceinline__ Limbs limbs_of(int64_t b) {
 __host__ __device__ __forceinline__ Limbs limbs_of(const int32_t (&b)[2]) { return {b[0], b[1]}; }
 // a b / 2^63 to about one unit: the products of the low limbs are left out and their
 // mean (1/4), together with half a unit for rounding, is added as CENTRED 2^-31 (the mean
-// error is then zero; zero times anything is zero). |a|, |b| < 2^62, or a < 2^63 beside
-// |b| < 2^61.
+// error is then zero; zero times anything is zero). |a|, |b| < 2^62, or |a| < 2^63
+// beside |b| <= 2^63 / 3.
 constexpr uint32_t CENTRED = 3u << 29;
 __host__ __device__ __forceinline__ int64_t mul63(int64_t a, Limbs b) {
   const int32_t ah = int32_t(a >> 32), al = int32_t(uint32_t(a) >> 1);
@@ -86,6 +86,18 @@ __host__ __device__ __forceinline__ bool fixed_in_range(const double (&h)[19], c
   for (int k = 6; k < 18; ++k) diag = diag > s(k) ? diag : s(k);
   // sum < (6/32 + 12/64 + 1/8) S = S / 2; rest >= S / 64
   return axis < 7u && diag < 6u && s(18) - 6u < 3u;
+}
+
+// The same windows for closed populations (S 2^-12 is 2^52): positive, and no larger.
+__host__ __device__ __forceinline__ bool fixed_closed_in_range(const int64_t (&f)[19]) {
+  auto top = [&](int k) { return uint32_t(uint64_t(f[k]) >> 32) - (1u << 20); };
+  uint32_t axis = 0, diag = 0;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) axis = axis > top(k) ? axis : top(k);
+#pragma unroll
+  for (int k = 6; k < 18; ++k) diag = diag > top(k) ? diag : top(k);
+  const uint32_t rest = uint32_t(uint64_t(f[18]) >> 32) - (1u << 26);
+  return axis < (1u << 27) - (1u << 20) && diag < (1u << 26) - (1u << 20) && rest < (1u << 29) - (1u << 26);
 }
 
 __host__ __device__ __forceinline__ int64_t fixed_in(double v, const FixedArgs& fx) {

@@ -677,6 +677,10 @@ __device__ __forceinline__ void apply_rule(uint32_t r, T (&h)[Q], Wide<T> ref) {
   }
 }
 
+}  // namespace lbm
+#include "fixed_close.cuh"
+namespace lbm {
+
 // Density deviation, velocity, and BGK relaxation toward the second-order
 // equilibrium (eq. rho, eq. vel, eq. feq, eq. bgk) on shifted populations:
 //   h_i^eq = w_i (drho + rho (3 c.u + 9/2 (c.u)^2 - 3/2 u^2)).
@@ -1029,29 +1033,10 @@ __device__ __forceinline__ void close_node(const SweepArgs& a, uint32_t lm, int 
   }
 }
 
-// Moments, residual terms and relaxation of one node on its closed populations. FP64
-// nodes whose populations lie in the windows of fixed64.cuh are relaxed there; with
-// RESID their density and velocity are the fixed-point sums rounded to double.
+// Moments, residual terms and relaxation of one node on its closed populations.
 template <typename S, bool RESID, bool GEOM, typename T>
 __device__ __forceinline__ void relax_node(const SweepArgs& a, T (&h)[Q], uint32_t cell, bool solid, NodeTerms<T>& terms) {
   T* snap = static_cast<T*>(a.snap);
-  if constexpr (std::is_same<T, double>::value) {
-    if (a.fx.on && !solid && fixed_in_range(h, a.fx)) {
-      int64_t f[Q];
-      FixedSums q = fixed_sums_of(h, a.fx, f);
-      if constexpr (RESID)
-        terms = residual_terms(moments_of(q, a.fx, GEOM && a.forced ? a.force : nullptr), snap, a.N, cell);
-      if constexpr (GEOM) {
-        if (a.forced) {
-          q.x += a.fx.force[0];
-          q.y += a.fx.force[1];
-          q.z += a.fx.force[2];
-        }
-      }
-      fixed_relax(f, q, a.fx, h);
-      return;
-    }
-  }
   Moments<T> m;
   if constexpr (GEOM && std::is_same<S, float>::value) m = moments_compensated(h, rho0_of<T>(a));
   else m = moments(h, rho0_of<T>(a));
@@ -1083,6 +1068,48 @@ __device__ __forceinline__ void relax_node(const SweepArgs& a, T (&h)[Q], uint32
     terms = residual_terms(m, snap, a.N, cell);
   }
   if (!solid) collide<std::is_same<S, float>::value>(h, m, omega_of<T>(a), a.mom_coef);
+}
+
+// Closure and relaxation of an FP64 node in fixed point; false, with h unchanged in no
+// particular way, where the node has to be taken in double.
+template <bool RESID, bool GEOM>
+__device__ __forceinline__ bool update_fixed(const SweepArgs& a, uint32_t lm, int code, uint32_t x, uint32_t y, uint32_t z,
+                                             uint32_t cell, double (&h)[Q], NodeTerms<double>& terms) {
+  if (GEOM && (lm & SOLID_NODE)) return false;
+  if (code != 0 && (!GEOM || ((lm >> RULE_SHIFT) & RULE_BITS) == 0u)) fixed_fill_unknown(a, code, h);
+  if (!fixed_in_range(h, a.fx)) return false;
+  int64_t f[Q];
+  static_for<0, Q>([&](auto kc) { f[decltype(kc)::value] = fixed_in(h[decltype(kc)::value], a.fx); });
+  if (!fixed_close_node<GEOM>(a, lm, code, x, y, z, f)) return false;
+  FixedSums q = fixed_sums(f);
+  if constexpr (RESID)
+    terms = residual_terms(moments_of(q, a.fx, GEOM && a.forced ? a.force : nullptr), static_cast<double*>(a.snap), a.N, cell);
+  if constexpr (GEOM) {
+    if (a.forced) {
+      q.x += a.fx.force[0];
+      q.y += a.fx.force[1];
+      q.z += a.fx.force[2];
+    }
+  }
+  fixed_relax(f, q, a.fx, h);
+  return true;
+}
+
+// One node: load(h) fetches its streamed populations, on return h holds the new ones. FP64
+// nodes go through fixed point where they can; the few others are loaded again, which
+// keeps their doubles from occupying registers meanwhile.
+template <typename S, bool RESID, bool GEOM, typename T, typename Load>
+__device__ __forceinline__ void update_node(const SweepArgs& a, uint32_t lm, int code, uint32_t x, uint32_t y, uint32_t z,
+                                            uint32_t cell, Load&& load, T (&h)[Q], NodeTerms<T>& terms) {
+  load(h);
+  if constexpr (std::is_same<T, double>::value) {
+    if (a.fx.on) {
+      if (update_fixed<RESID, GEOM>(a, lm, code, x, y, z, cell, h, terms)) return;
+      load(h);
+    }
+  }
+  close_node<GEOM>(a, lm, code, x, y, z, h);
+  relax_node<S, RESID, GEOM>(a, h, cell, (lm & SOLID_NODE) != 0u, terms);
 }
 
 // ---------------------------------------------------------------------------------
@@ -1134,39 +1161,39 @@ __device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk) {
     // geometry word (A/B lattices with a geometry only; 0 everywhere else)
     uint32_t lm = 0u;
     if constexpr (GEOM) lm = a.links ? __ldg(a.links + chk(cell, a.N)) : 0u;
-    T h[Q];
-    if (!GEOM || (lm & ~(RULE_BITS << RULE_SHIFT)) == 0u) {
-      static_for<0, Q>([&](auto kc) {
-        constexpr int k = decltype(kc)::value;
-        if constexpr (MODE == STREAM_AB) {
-          h[k] = Storage<S>::load(static_cast<const S*>(a.src_pop[k]) + pull_idx(kc));
-        } else if constexpr (MODE == STREAM_AA_GATHER) {
-          h[k] = load_pop<S, MODE>(static_cast<const S*>(a.src_pop[opp(k)]) + pull_idx(kc));
-        } else {
-          h[k] = load_pop<S, MODE>(static_cast<const S*>(a.src_pop[k]) + cell);
-        }
-      });
-    } else {
-      // a solid node keeps its populations; next to a solid node the population that
-      // would come from it is the node's own population -k reversed (mid-grid
-      // bounce-back, Sec. "Boundary conditions")
-      static_for<0, Q>([&](auto kc) {
-        constexpr int k = decltype(kc)::value;
-        const bool own = (lm & SOLID_NODE) != 0u;
-        const bool back = (lm >> k) & 1u;
-        const S* p = own ? static_cast<const S*>(a.src_pop[k]) + cell
-                         : (back ? static_cast<const S*>(a.src_pop[opp(k)]) + cell
-                                 : static_cast<const S*>(a.src_pop[k]) + pull_idx(kc));
-        h[k] = Storage<S>::load(p);
-      });
-    }
-    const bool solid = (lm & SOLID_NODE) != 0u;
+    auto load = [&](T (&h)[Q]) {
+      if (!GEOM || (lm & ~(RULE_BITS << RULE_SHIFT)) == 0u) {
+        static_for<0, Q>([&](auto kc) {
+          constexpr int k = decltype(kc)::value;
+          if constexpr (MODE == STREAM_AB) {
+            h[k] = Storage<S>::load(static_cast<const S*>(a.src_pop[k]) + pull_idx(kc));
+          } else if constexpr (MODE == STREAM_AA_GATHER) {
+            h[k] = load_pop<S, MODE>(static_cast<const S*>(a.src_pop[opp(k)]) + pull_idx(kc));
+          } else {
+            h[k] = load_pop<S, MODE>(static_cast<const S*>(a.src_pop[k]) + cell);
+          }
+        });
+      } else {
+        // a solid node keeps its populations; next to a solid node the population that
+        // would come from it is the node's own population -k reversed (mid-grid
+        // bounce-back, Sec. "Boundary conditions")
+        static_for<0, Q>([&](auto kc) {
+          constexpr int k = decltype(kc)::value;
+          const bool own = (lm & SOLID_NODE) != 0u;
+          const bool back = (lm >> k) & 1u;
+          const S* p = own ? static_cast<const S*>(a.src_pop[k]) + cell
+                           : (back ? static_cast<const S*>(a.src_pop[opp(k)]) + cell
+                                   : static_cast<const S*>(a.src_pop[k]) + pull_idx(kc));
+          h[k] = Storage<S>::load(p);
+        });
+      }
+    };
     const int fx = px ? 0 : (x == 0 ? 1 : (x == a.nx - 1 ? 2 : 0));
     const int fy = py ? 0 : (y == 0 ? 1 : (y == a.ny - 1 ? 2 : 0));
     const int fz = pz ? 0 : (z == 0 ? 1 : (z == a.nz - 1 ? 2 : 0));
     const int code = fx + 3 * fy + 9 * fz;
-    close_node<GEOM>(a, lm, code, x, y, z, h);
-    relax_node<S, RESID, GEOM>(a, h, cell, solid, terms);
+    T h[Q];
+    update_node<S, RESID, GEOM>(a, lm, code, x, y, z, cell, load, h, terms);
     static_for<0, Q>([&](auto kc) {
       constexpr int k = decltype(kc)::value;
       if constexpr (MODE == STREAM_AB) {

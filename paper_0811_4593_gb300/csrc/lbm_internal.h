@@ -39,8 +39,8 @@ inline float floor_neg(double rho0) {
   return double(f) > -rho0 ? std::nextafter(f, -INFINITY) : f;
 }
 
-// One boundary-face node as the sweep reads it, the first half by FP64 sweeps, the second
-// by float ones. Velocity face: the prescribed velocity and 1 / (1 - u.n) for the density
+// One boundary-face node as the sweep reads it: the first half for FP64 arithmetic, the
+// second for float sweeps, or in an FP64 lattice for its fixed-point closures. Velocity face: the prescribed velocity and 1 / (1 - u.n) for the density
 // relation (n = inward normal), formed in double on the host, for float sweeps as a pair
 // hi + lo. Pressure face: the tangential velocity (normal part zero), the prescribed
 // density in `inv`, and for float sweeps its reciprocal as a pair, the density and its
@@ -48,10 +48,15 @@ inline float floor_neg(double rho0) {
 struct __align__(16) FaceNode {
   double u[3];
   double inv;
-  float uf[3];
-  float inv_hi, inv_lo;
-  float rho, drho;
-  float pad;
+  union {
+    struct {
+      float uf[3];
+      float inv_hi, inv_lo;
+      float rho, drho;
+      float pad;
+    };
+    int64_t fx[4];  // FixedFace: u[0], u[1], r, ok (make_fixed_face)
+  };
 };
 
 // Boundary data of one face for the sweep.
@@ -71,6 +76,7 @@ struct FixedArgs {
   int32_t w[2];       // omega / 36
   int64_t force[3];   // tau F in units of S 2^-64
   double unit_in, unit_out;  // S 2^-64, S 2^-63
+  double rest[2];     // axis and diagonal populations at rest: rho0 / 18, rho0 / 36
 };
 
 // The parameters for density scale rho0, omega and tau F. Off where a scale has no
@@ -99,8 +105,35 @@ inline FixedArgs make_fixed(double rho0, double omega, const double (&tforce)[3]
   fx.e_out = uint32_t(991 + e) << 20;
   fx.unit_in = std::ldexp(1.0, e - 64);
   fx.unit_out = std::ldexp(1.0, e - 63);
+  fx.rest[0] = rho0 / 18.0;
+  fx.rest[1] = rho0 / 36.0;
   fx.on = 1u;
   return fx;
+}
+
+// The fixed-point record of a face node on axis `axis` with inward normal component un and
+// velocity u (velocity face), or density rho (pressure face). Marked unfit (0) where the
+// velocity is not below 1/4 or the density not near the lattice's, and in lattices that
+// relax in double.
+inline void make_fixed_face(const FixedArgs& fx, int axis, const double* u, double un, bool pressure, double rho,
+                            int64_t (&out)[4]) {
+  out[0] = out[1] = out[2] = out[3] = 0;
+  if (!fx.on) return;
+  int n = 0;
+  for (int i = 0; i < 3; ++i) {
+    if (i == axis) continue;
+    if (!(std::fabs(u[i]) < 0.25)) return;
+    out[n++] = std::llrint(std::ldexp(u[i] * 2.0 / 3.0, 62));
+  }
+  if (pressure) {
+    const double r = rho / fx.unit_in;  // S is a power of two
+    if (!(r > 0x1p60) || !(r < 0x1p63)) return;
+    out[2] = int64_t(r);
+  } else {
+    if (!(std::fabs(un) < 0.25)) return;
+    out[2] = std::llrint(std::ldexp(un / (1.0 - un), 62));  // 1 / (1 - un) - 1
+  }
+  out[3] = 1;
 }
 
 // Everything one sweep launch needs, passed by value.

@@ -97,11 +97,11 @@ __global__ void __launch_bounds__(RESIDENT_THREADS, 1)
     if (active) {
       const uint32_t array = (s & 1) ? array_bytes : 0u;
       T h[Q];
-      static_for<0, Q>([&](auto kc) { h[decltype(kc)::value] = ld_cluster(from[decltype(kc)::value] + array, S()); });
-      const bool solid = (lm & SOLID_NODE) != 0u;
-      close_node<GEOM>(a, lm, code, x, y, z, h);
+      auto load = [&](T (&v)[Q]) {
+        static_for<0, Q>([&](auto kc) { v[decltype(kc)::value] = ld_cluster(from[decltype(kc)::value] + array, S()); });
+      };
       NodeTerms<T> unused;
-      relax_node<S, false, GEOM>(a, h, cell, solid, unused);
+      update_node<S, false, GEOM>(a, lm, code, x, y, z, cell, load, h, unused);
       if (last) {
         static_for<0, Q>([&](auto kc) {
           constexpr int k = decltype(kc)::value;

@@ -182,13 +182,18 @@ void ctx_free_all(lbm_ctx* ctx) {
 // Sweep record of one node of face f. Velocity face: u and 1 / (1 - u.n) (n the inward
 // normal; |u.n| < 1 is validated). Pressure face: the tangential part of u and the
 // prescribed density (see FaceNode).
-lbm::FaceNode face_node(int f, const double* u, bool pressure, double rho, double rho0) {
+lbm::FaceNode face_node(int f, const double* u, bool pressure, double rho, double rho0, bool f64,
+                        const lbm::FixedArgs& fx) {
   lbm::FaceNode n{};
   for (int j = 0; j < 3; ++j) n.u[j] = (pressure && j == f / 2) ? 0.0 : u[j];
-  for (int j = 0; j < 3; ++j) n.uf[j] = float(n.u[j]);
   const double un = (f % 2 == 0 ? 1.0 : -1.0) * u[f / 2];
   const double inv = pressure ? 1.0 / rho : 1.0 / (1.0 - un);
   n.inv = pressure ? rho : inv;
+  if (f64) {
+    lbm::make_fixed_face(fx, f / 2, n.u, un, pressure, rho, n.fx);
+    return n;
+  }
+  for (int j = 0; j < 3; ++j) n.uf[j] = float(n.u[j]);
   n.inv_hi = float(inv);
   n.inv_lo = float(inv - double(n.inv_hi));
   n.rho = float(rho);
@@ -500,7 +505,7 @@ lbm_status lbm_create_scheme(int nx, int ny, int nz, double tau, const lbm_face_
     const bool pres = faces[f].kind == LBM_FACE_PRESSURE;
     if (pres) a.pressure |= 1u << f;
     a.face[f].tab = nullptr;
-    a.face[f].uni = face_node(f, open ? faces[f].u : zero, pres, pres ? faces[f].rho : 0.0, rho0);
+    a.face[f].uni = face_node(f, open ? faces[f].u : zero, pres, pres ? faces[f].rho : 0.0, rho0, prec == LBM_F64, a.fx);
     const bool per_node = open && (faces[f].u_table || (pres && faces[f].rho_table));
     if (per_node) {
       const size_t m = size_t(face_n1(f, nx, ny)) * face_n2(f, ny, nz);
@@ -508,7 +513,7 @@ lbm_status lbm_create_scheme(int nx, int ny, int nz, double tau, const lbm_face_
       for (size_t i = 0; i < m; ++i) {
         const double* u = faces[f].u_table ? faces[f].u_table + 3 * i : faces[f].u;
         const double r = pres ? (faces[f].rho_table ? faces[f].rho_table[i] : faces[f].rho) : 0.0;
-        host[i] = face_node(f, u, pres, r, rho0);
+        host[i] = face_node(f, u, pres, r, rho0, prec == LBM_F64, a.fx);
       }
       const size_t bytes = m * sizeof(lbm::FaceNode);
       void* t = ctx_alloc(ctx, bytes);
@@ -743,7 +748,9 @@ lbm_status lbm_set_geometry(lbm_ctx* ctx, const uint8_t* solid, const int8_t* co
                       "node (%d, %d, %d): code %d leaves a population from a solid or outside node unset", x,
                       y, z, c);
         const uint32_t rule = c > 0 ? uint32_t(c) : uint32_t(44 - c);
-        links[node] = rule << lbm::RULE_SHIFT;
+        // the unknown populations are loaded as the node's own reversed ones and then
+        // overwritten (a solid source may hold anything)
+        links[node] = (rule << lbm::RULE_SHIFT) | rule_mask;
       }
   if (!ctx->args.links) {
     void* d = ctx_alloc(ctx, sizeof(uint32_t) * ctx->N);

@@ -67,3 +67,49 @@ def test_one_step_matches_the_oracle(rho0, tau, mix):
     size = np.abs(streamed).sum(0)
     grow = np.maximum(1.0, size / np.maximum(np.abs(streamed.sum(0)), 1e-300)) ** 2
     assert np.all(np.abs(got - ref) <= 60 * 2.0 ** -53 * size * grow)
+
+
+def _solid():
+    wl = inp.channel(19, 16, 17, 0.9, (0.03, 0.01, 0.0))
+    wl.solid = (inp.noise(5, (17, 16, 19)) > 0.6).astype(np.uint8)
+    return wl
+
+
+CLOSURES = {
+    "faces": lambda: inp.random_face_workload(51, 13, 10, 9, 0.8, (False, False, False)),
+    "faces_beyond_a_quarter": lambda: inp.random_face_workload(52, 13, 10, 9, 1.0, (False, False, False), amp=0.4),
+    "x_rows_of_three": lambda: inp.random_face_workload(53, 3, 17, 11, 0.9, (False, True, False)),
+    "pressure": lambda: inp.random_pressure_workload(54, 12, 9, 11, 0.9),
+    "pressure_far_off": lambda: inp.random_pressure_workload(55, 12, 9, 11, 0.9, periodic_y=True, amp=0.9),
+    "embedded": lambda: inp.embedded_walls(inp.make_workload("box", 9, 8, 7, 0.8, [inp.ZERO] * 6)),
+    "pillar_x": lambda: inp.pillar_channel(axis=0, flow=1),
+    "pillar_y": lambda: inp.pillar_channel(axis=1, flow=0),
+    "pillar_z": lambda: inp.pillar_channel(axis=2, flow=1, force=3e-3),
+    "solid": _solid,
+}
+
+
+@pytest.mark.parametrize("mix", [False, True])
+@pytest.mark.parametrize("name", list(CLOSURES))
+def test_closures_match_the_oracle(name, mix):
+    # every face, edge, corner and geometry rule, with prescribed values on both sides of
+    # what the fixed-point closures take, on states inside and partly outside the windows
+    import oracle
+    import paper_0811_4593_gb300 as lbm
+    wl = CLOSURES[name]()
+    shape = (19, wl.nz, wl.ny, wl.nx)
+    w = oracle.lattice()[1][:, None, None, None]
+    f0 = w * (1.0 + 0.1 * inp.noise(21, shape))
+    if mix:
+        f0 *= np.exp2(-2.0 + 3.0 * inp.noise(22, shape)) ** (inp.noise(23, shape) > 0.9)
+    with lbm.Lattice.from_workload(wl, "f64") as lat:
+        lat.set_populations(f0)
+        lat.step(1)
+        got = lat.get_populations()
+        lat.check_guards()
+    ref = oracle.run(oracle.Lattice.from_workload(wl), f0, 1)
+    # about 100 roundings of numbers no larger than the neighbourhood's populations, times
+    # 1 / (1 - u.n) <= 5/3 of a closure and its square in the equilibrium; a pressure plane
+    # of density 0.1 next to density 1 has |u| near 1, squared over 0.1
+    size = max(np.abs(f0).sum(0).max(), np.abs(ref).sum(0).max())
+    assert np.abs(got - ref).max() <= 100 * 2.0 ** -53 * size * (10.0 if "far" in name else 3.0)
