@@ -114,9 +114,14 @@ __device__ __forceinline__ uint32_t chk(uint32_t i, uint32_t) { return i; }
 // it has completed and its stores are visible. `index` ties every address to the wait:
 // loads written as plain functions of a pointer may otherwise be moved above it. Without
 // such a launch both instructions do nothing.
-__device__ __forceinline__ void wait_for_previous_sweep(uint32_t& index) {
+// `ahead`: a value that no sweep writes, loaded before the wait.
+__device__ __forceinline__ void wait_for_previous_sweep(uint32_t& index, uint32_t& ahead) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" : "+r"(index)::"memory");
+  asm volatile("griddepcontrol.wait;" : "+r"(index), "+r"(ahead)::"memory");
+}
+__device__ __forceinline__ void wait_for_previous_sweep(uint32_t& index) {
+  uint32_t none = 0;
+  wait_for_previous_sweep(index, none);
 }
 
 // Signed sums whose first term is taken as it is (negation is exact), so that no
@@ -151,6 +156,19 @@ __host__ __device__ constexpr int first_with(int a, int sg) {
     const int c = ca(k, a);
     if ((sg > 0 && c > 0) || (sg < 0 && c < 0) || (sg == 0 && c == 0)) return k;
   }
+  return -1;
+}
+// Population k with c_x reversed.
+__host__ __device__ constexpr int mirror_x(int k) { return vel_index(-cx(k), cy(k), cz(k)); }
+// how many populations below k have a component a, and the n-th that has one
+__host__ __device__ constexpr int rank_with(int a, int k) {
+  int n = 0;
+  for (int i = 0; i < k; ++i) n += ca(i, a) != 0;
+  return n;
+}
+__host__ __device__ constexpr int nth_with(int a, int n) {
+  for (int k = 0; k < Q; ++k)
+    if (ca(k, a) != 0 && n-- == 0) return k;
   return -1;
 }
 __host__ __device__ constexpr int first_nonzero(int a) {
@@ -213,6 +231,15 @@ __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float t) {
   const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(t, bb));
   hi = s;
   lo = __fadd_rn(lo, e);
+}
+
+// The same on two sums at once.
+__device__ __forceinline__ void two_sum_acc(f32x2& hi, f32x2& lo, f32x2 t) {
+  const f32x2 s = op_add(hi, t);
+  const f32x2 bb = op_sub(s, hi);
+  const f32x2 e = op_add(op_sub(hi, op_sub(s, bb)), op_sub(t, bb));
+  hi = s;
+  lo = op_add(lo, e);
 }
 
 // A number of the density relations: double in FP64 sweeps, a float pair (about 47 bits)
@@ -482,9 +509,6 @@ __device__ __forceinline__ void face_case(const SweepArgs& a, uint32_t x, uint32
   else close_face<A, SG>(h, fv, ref_density<T>(a));
 }
 
-// Population k with c_x reversed.
-__host__ __device__ constexpr int mirror_x(int k) { return vel_index(-cx(k), cy(k), cz(k)); }
-
 // Both x faces in one body: a node of the high face is mirrored in x, closed as one of
 // the low face and mirrored back. Warps of short rows hold nodes of both faces and would
 // run the body twice. The mirrored sums take their terms in the same order, so the bits
@@ -724,16 +748,20 @@ __device__ __forceinline__ Moments<T> moments(const T (&h)[Q], T rho0) {
 // and integrate over the relaxation time (a 32^3 body-force Poiseuille at tau = 2
 // relaxes over ~190 steps), so the exact sums reduce the float error of such flows.
 __device__ __forceinline__ Moments<float> moments_compensated(const float (&h)[Q], float rho0) {
-  float sp = 0.0f, spl = 0.0f, sm = 0.0f, sml = 0.0f, s0 = 0.0f, s0l = 0.0f;
-  float jy = 0.0f, jyl = 0.0f, jz = 0.0f, jzl = 0.0f;
+  // the c_x = +1 and -1 sums side by side as packed pairs, and so the y and z momenta
+  f32x2 p(0.0f), pl(0.0f), q(0.0f), ql(0.0f);
+  float s0 = 0.0f, s0l = 0.0f;
   static_for<0, Q>([&](auto kc) {
     constexpr int k = decltype(kc)::value;
-    if constexpr (cx(k) > 0) two_sum_acc(sp, spl, h[k]);
-    else if constexpr (cx(k) < 0) two_sum_acc(sm, sml, h[k]);
-    else two_sum_acc(s0, s0l, h[k]);
-    if constexpr (cy(k) != 0) two_sum_acc(jy, jyl, cy(k) > 0 ? h[k] : -h[k]);
-    if constexpr (cz(k) != 0) two_sum_acc(jz, jzl, cz(k) > 0 ? h[k] : -h[k]);
+    if constexpr (cx(k) > 0) two_sum_acc(p, pl, f32x2(h[k], h[mirror_x(k)]));
+    if constexpr (cx(k) == 0) two_sum_acc(s0, s0l, h[k]);
+    // the i-th population with c_y != 0 beside the i-th with c_z != 0
+    if constexpr (cy(k) != 0) {
+      constexpr int z = nth_with(2, rank_with(1, k));
+      two_sum_acc(q, ql, f32x2(cy(k) > 0 ? h[k] : -h[k], cz(z) > 0 ? h[z] : -h[z]));
+    }
   });
+  const float sp = p.x, spl = pl.x, sm = p.y, sml = pl.y, jy = q.x, jyl = ql.x, jz = q.y, jzl = ql.y;
   Moments<float> m;
   float d = sp, dl = __fadd_rn(__fadd_rn(spl, sml), s0l);
   two_sum_acc(d, dl, sm);
@@ -1112,6 +1140,13 @@ __device__ __forceinline__ void update_node(const SweepArgs& a, uint32_t lm, int
   relax_node<S, RESID, GEOM>(a, h, cell, (lm & SOLID_NODE) != 0u, terms);
 }
 
+// Geometry word of node blk*256 + threadIdx.x (A/B lattices with a geometry; 0 everywhere
+// else).
+__device__ __forceinline__ uint32_t geometry_word(const SweepArgs& a, uint32_t blk) {
+  const uint32_t cell = blk * SWEEP_THREADS + threadIdx.x;
+  return a.links && cell < a.N ? __ldg(a.links + chk(cell, a.N)) : 0u;
+}
+
 // ---------------------------------------------------------------------------------
 // The fused time step: pull stream, classify, close, collide, store.
 // ---------------------------------------------------------------------------------
@@ -1127,12 +1162,14 @@ enum StreamMode : int { STREAM_AB = 0, STREAM_AA_GATHER = 1, STREAM_AA_LOCAL = 2
 // populations in natural slots, after the local step the swapped post-collision state
 // again. Each node reads and writes the same 19 locations, so one array suffices.
 // GEOM: the lattice may have a geometry (solid nodes, on-site rules) and a body force;
-// the plain variant reads neither.
+// the plain variant reads neither. `lm`: the thread's geometry word (geometry_word).
+// A solid node keeps its populations, and both arrays hold them (lbm_set_geometry,
+// lbm_set_populations), so a plain step neither reads nor writes it.
 template <typename S, bool RESID, int MODE, bool GEOM = false>
-__device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk) {
+__device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk, uint32_t lm = 0u) {
   using T = typename ComputeOf<S>::T;
   const uint32_t cell = blk * SWEEP_THREADS + threadIdx.x;
-  const bool active = cell < a.N;
+  const bool active = cell < a.N && (!GEOM || RESID || !(lm & SOLID_NODE));
   NodeTerms<T> terms = {};
   if (active) {
     const uint32_t q1 = fdiv(a.div_nx, cell);
@@ -1158,9 +1195,6 @@ __device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk) {
       const uint32_t sz = cz(k) > 0 ? zm : (cz(k) < 0 ? zp : z);
       return chk((sz * a.ny + sy) * a.nx + sx, a.N);
     };
-    // geometry word (A/B lattices with a geometry only; 0 everywhere else)
-    uint32_t lm = 0u;
-    if constexpr (GEOM) lm = a.links ? __ldg(a.links + chk(cell, a.N)) : 0u;
     auto load = [&](T (&h)[Q]) {
       if (!GEOM || (lm & ~(RULE_BITS << RULE_SHIFT)) == 0u) {
         static_for<0, Q>([&](auto kc) {
@@ -1240,8 +1274,16 @@ template <typename S, bool RESID, int MODE, bool GEOM>
 __global__ void __launch_bounds__(SWEEP_THREADS, (SweepOccupancy<S, RESID, false, MODE, GEOM>::blocks))
     sweep_kernel(const __grid_constant__ SweepArgs a) {
   uint32_t blk = blockIdx.x;
-  wait_for_previous_sweep(blk);
-  sweep_block<S, RESID, MODE, GEOM>(a, blk);
+  if constexpr (GEOM) {
+    // the geometry does not change between sweeps: its word is on its way (or here) when
+    // the previous sweep ends, so the population loads do not wait for it
+    uint32_t lm = geometry_word(a, blk);
+    wait_for_previous_sweep(blk, lm);
+    sweep_block<S, RESID, MODE, GEOM>(a, blk, lm);
+  } else {
+    wait_for_previous_sweep(blk);
+    sweep_block<S, RESID, MODE, GEOM>(a, blk);
+  }
 }
 
 // ---------------------------------------------------------------------------------
@@ -1728,7 +1770,7 @@ __global__ void __launch_bounds__(SWEEP_THREADS, (SweepOccupancy<S, RESID, true,
         __syncthreads();
       }
       if constexpr (MODE == STREAM_AB) {
-        if (sa.links || sa.forced) sweep_block<S, RESID, MODE, true>(sa, b - lat_begin);
+        if (sa.links || sa.forced) sweep_block<S, RESID, MODE, true>(sa, b - lat_begin, geometry_word(sa, b - lat_begin));
         else sweep_block<S, RESID, MODE, false>(sa, b - lat_begin);
       } else {
         sweep_block<S, RESID, MODE, false>(sa, b - lat_begin);

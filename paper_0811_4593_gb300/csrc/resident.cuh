@@ -54,10 +54,13 @@ __global__ void __launch_bounds__(RESIDENT_THREADS, 1)
   S* const buf = reinterpret_cast<S*>(resident_smem);  // [2][19][per]
   const uint32_t per = blockDim.x, tid = threadIdx.x;
   const uint32_t cell = blockIdx.x * per + tid;
-  const bool active = cell < a.N;
+  uint32_t lm = 0;
+  if (GEOM && a.links && cell < a.N) lm = __ldg(a.links + cell);
+  // solid nodes keep their populations, in both global arrays, and nobody reads them
+  const bool active = cell < a.N && !(lm & SOLID_NODE);
   const uint32_t array_bytes = Q * per * uint32_t(sizeof(S));
   uint32_t from[Q];  // shared-window addresses of the pull sources in array 0
-  uint32_t x = 0, y = 0, z = 0, lm = 0;
+  uint32_t x = 0, y = 0, z = 0;
   int code = 0;
   if (active) {
     const uint32_t q1 = fdiv(a.div_nx, cell);
@@ -72,7 +75,6 @@ __global__ void __launch_bounds__(RESIDENT_THREADS, 1)
     const int fy = py ? 0 : (y == 0 ? 1 : (y == a.ny - 1 ? 2 : 0));
     const int fz = pz ? 0 : (z == 0 ? 1 : (z == a.nz - 1 ? 2 : 0));
     code = fx + 3 * fy + 9 * fz;
-    if constexpr (GEOM) lm = a.links ? __ldg(a.links + chk(cell, a.N)) : 0u;
     const bool links = GEOM && (lm & ~(RULE_BITS << RULE_SHIFT)) != 0u;
     static_for<0, Q>([&](auto kc) {
       constexpr int k = decltype(kc)::value;
@@ -81,10 +83,7 @@ __global__ void __launch_bounds__(RESIDENT_THREADS, 1)
       const uint32_t sz = cz(k) > 0 ? zm : (cz(k) < 0 ? zp : z);
       uint32_t source = chk((sz * a.ny + sy) * a.nx + sx, a.N);
       uint32_t slot = k;
-      if (links) {  // a solid node keeps its populations, a solid source sends the node's own back
-        if (lm & SOLID_NODE) source = cell;
-        else if ((lm >> k) & 1u) source = cell, slot = opp(k);
-      }
+      if (links && ((lm >> k) & 1u)) source = cell, slot = opp(k);  // a solid source sends the node's own back
       const uint32_t rank = source / per;
       from[k] = cluster_address(smem_u32(buf + slot * per + (source - rank * per)), rank);
       const S* own = static_cast<const S*>(a.src_pop[swapped ? opp(k) : k]);

@@ -641,6 +641,10 @@ static lbm_status copy_populations(lbm_ctx* ctx, void* host_or_dev, int z0, int 
     char* l = lat + (size_t(slot) * ctx->N + size_t(z0) * plane) * es;
     char* u = user + size_t(k) * slab;
     LBM_CUDA(ctx, cudaMemcpyAsync(to_ctx ? l : u, to_ctx ? u : l, slab, kind, ctx->stream), "population copy");
+    // plain steps leave solid nodes alone in both arrays: the other one takes them too
+    if (to_ctx && ctx->args.links)
+      LBM_CUDA(ctx, cudaMemcpyAsync(static_cast<char*>(ctx->buf[ctx->cur ^ 1]) + (l - lat), l, slab,
+                                    cudaMemcpyDeviceToDevice, ctx->stream), "population copy");
   }
   LBM_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "synchronising the population copy");
   return to_ctx ? LBM_OK : check_device_error(ctx);
@@ -759,7 +763,8 @@ lbm_status lbm_set_geometry(lbm_ctx* ctx, const uint8_t* solid, const int8_t* co
   }
   LBM_CUDA(ctx, cudaMemcpyAsync(const_cast<uint32_t*>(ctx->args.links), links.data(), sizeof(uint32_t) * ctx->N,
                                 cudaMemcpyHostToDevice, ctx->stream), "uploading the geometry words");
-  // solid nodes are carried unchanged from buffer to buffer: start both alike
+  // solid nodes keep their populations, and plain steps leave them alone in both arrays:
+  // start both alike
   LBM_CUDA(ctx, cudaMemcpyAsync(ctx->buf[ctx->cur ^ 1], ctx->buf[ctx->cur], 19ull * ctx->N * storage_bytes(ctx->prec),
                                 cudaMemcpyDeviceToDevice, ctx->stream), "copying the state");
   LBM_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "synchronising");
