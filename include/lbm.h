@@ -144,9 +144,12 @@ LBM_API lbm_status lbm_set_stream(lbm_ctx* ctx, void* cuda_stream);
  * the edge correction eq. edge, buried links eq. buried and eq. corner; then BGK
  * collision (eq. bgk, eq. feq). Binary16 lattices whose rows are multiples of 8 nodes
  * and at least 256 long take a sweep that stages population rows in shared memory with
- * bulk copies; its waits are bounded, and one that runs out is reported by the next
- * synchronising call as LBM_ERR_CUDA (see lbm_debug_drop_staged_copies). Every sweep
- * variant computes the same bits for a node. */
+ * bulk copies. 16 or more steps of a small lattice are one launch: up to 8,192 nodes (FP64
+ * 4,096) of one thread-block cluster, A/B lattices beyond, up to 1,024 nodes per SM (FP64
+ * 512), of a cooperative grid with a barrier between steps. Waits of either kind of kernel
+ * are bounded, and one that runs out is reported by the next synchronising call as
+ * LBM_ERR_CUDA (see lbm_debug_drop_staged_copies). Every sweep variant computes the same
+ * bits for a node. */
 LBM_API lbm_status lbm_step(lbm_ctx* ctx, int n);
 
 /* Advance n >= 1 steps like lbm_step, the last one also forming, in double, the
@@ -249,8 +252,9 @@ LBM_API lbm_status lbm_debug_bounds_errors(int* enabled, uint64_t* count);
  * of the steps since the previous such call is then not valid, but the context stays
  * usable (load a state with lbm_set_populations). With enable != 0, later row-staged
  * sweeps of `ctx` leave the copies of one row group un-issued, so that a wait runs
- * out on purpose (no fault: the sweep ends after about two seconds); enable = 0 turns
- * this off. Other sweep kernels ignore it. */
+ * out on purpose (no fault: the sweep ends after about two seconds), and later multi-step
+ * launches with a grid barrier keep one block's arrival from it, with the same effect;
+ * enable = 0 turns this off. Other sweep kernels ignore it. */
 LBM_API lbm_status lbm_debug_drop_staged_copies(lbm_ctx* ctx, int enable);
 
 /* Block the host until the context's stream is idle; reports asynchronous errors. */

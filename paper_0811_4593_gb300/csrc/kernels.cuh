@@ -214,6 +214,14 @@ load_pop(const S* p) {
   else return Storage<S>::load(p);
 }
 
+template <typename S, bool COHERENT>
+__device__ __forceinline__ typename std::conditional<std::is_same<S, double>::value, double, float>::type
+load_source(const S* p) {
+  if constexpr (!COHERENT) return Storage<S>::load(p);
+  else if constexpr (std::is_same<S, __half>::value) return __half2float(__ldcg(p));
+  else return __ldcg(p);
+}
+
 // The reference density the register values are shifted by: rho0, or 0 for FP64.
 template <typename S>
 __device__ __forceinline__ double ref_rho(double rho0) { return Storage<S>::shifted ? rho0 : 0.0; }
@@ -1140,10 +1148,8 @@ __device__ __forceinline__ void update_node(const SweepArgs& a, uint32_t lm, int
   relax_node<S, RESID, GEOM>(a, h, cell, (lm & SOLID_NODE) != 0u, terms);
 }
 
-// Geometry word of node blk*256 + threadIdx.x (A/B lattices with a geometry; 0 everywhere
-// else).
-__device__ __forceinline__ uint32_t geometry_word(const SweepArgs& a, uint32_t blk) {
-  const uint32_t cell = blk * SWEEP_THREADS + threadIdx.x;
+// Geometry word of a node (A/B lattices with a geometry; 0 everywhere else).
+__device__ __forceinline__ uint32_t geometry_word(const SweepArgs& a, uint32_t cell) {
   return a.links && cell < a.N ? __ldg(a.links + chk(cell, a.N)) : 0u;
 }
 
@@ -1151,8 +1157,7 @@ __device__ __forceinline__ uint32_t geometry_word(const SweepArgs& a, uint32_t b
 // The fused time step: pull stream, classify, close, collide, store.
 // ---------------------------------------------------------------------------------
 enum StreamMode : int { STREAM_AB = 0, STREAM_AA_GATHER = 1, STREAM_AA_LOCAL = 2 };
-// Block `blk` (nodes blk*256 .. blk*256+255) of the lattice described by `a`, with the
-// streaming scheme MODE:
+// Node `cell` of the lattice described by `a`, with the streaming scheme MODE:
 //   STREAM_AB         pull f_i(x) = src_i(x - c_i), store dst_i(x)          (two arrays)
 //   STREAM_AA_GATHER  read slot -i of node x - c_i, write f*_i back to slot i of node
 //                     x + c_i -- the location the read of -i came from   (one array)
@@ -1165,13 +1170,11 @@ enum StreamMode : int { STREAM_AB = 0, STREAM_AA_GATHER = 1, STREAM_AA_LOCAL = 2
 // the plain variant reads neither. `lm`: the thread's geometry word (geometry_word).
 // A solid node keeps its populations, and both arrays hold them (lbm_set_geometry,
 // lbm_set_populations), so a plain step neither reads nor writes it.
-template <typename S, bool RESID, int MODE, bool GEOM = false>
-__device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk, uint32_t lm = 0u) {
-  using T = typename ComputeOf<S>::T;
-  const uint32_t cell = blk * SWEEP_THREADS + threadIdx.x;
-  const bool active = cell < a.N && (!GEOM || RESID || !(lm & SOLID_NODE));
-  NodeTerms<T> terms = {};
-  if (active) {
+// COHERENT: the source array is written by other blocks of the same launch (between grid
+// barriers), so it is read through L2.
+template <typename S, bool RESID, int MODE, bool GEOM = false, bool COHERENT = false, typename T>
+__device__ __forceinline__ void sweep_node(const SweepArgs& a, uint32_t cell, uint32_t lm, NodeTerms<T>& terms) {
+  if (cell < a.N && (!GEOM || RESID || !(lm & SOLID_NODE))) {
     const uint32_t q1 = fdiv(a.div_nx, cell);
     const uint32_t x = cell - q1 * a.nx;
     const uint32_t z = fdiv(a.div_ny, q1);
@@ -1200,7 +1203,7 @@ __device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk, ui
         static_for<0, Q>([&](auto kc) {
           constexpr int k = decltype(kc)::value;
           if constexpr (MODE == STREAM_AB) {
-            h[k] = Storage<S>::load(static_cast<const S*>(a.src_pop[k]) + pull_idx(kc));
+            h[k] = load_source<S, COHERENT>(static_cast<const S*>(a.src_pop[k]) + pull_idx(kc));
           } else if constexpr (MODE == STREAM_AA_GATHER) {
             h[k] = load_pop<S, MODE>(static_cast<const S*>(a.src_pop[opp(k)]) + pull_idx(kc));
           } else {
@@ -1218,7 +1221,7 @@ __device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk, ui
           const S* p = own ? static_cast<const S*>(a.src_pop[k]) + cell
                            : (back ? static_cast<const S*>(a.src_pop[opp(k)]) + cell
                                    : static_cast<const S*>(a.src_pop[k]) + pull_idx(kc));
-          h[k] = Storage<S>::load(p);
+          h[k] = load_source<S, COHERENT>(p);
         });
       }
     };
@@ -1245,6 +1248,14 @@ __device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk, ui
       }
     });
   }
+}
+
+// Block `blk` (nodes blk*256 .. blk*256+255).
+template <typename S, bool RESID, int MODE, bool GEOM = false>
+__device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk, uint32_t lm = 0u) {
+  using T = typename ComputeOf<S>::T;
+  NodeTerms<T> terms = {};
+  sweep_node<S, RESID, MODE, GEOM>(a, blk * SWEEP_THREADS + threadIdx.x, lm, terms);
   if constexpr (RESID)
     block_terms(terms, a.N, blk, ref_rho<S>(a.rho0), a.neg_rho0, static_cast<T*>(a.snap), a.partials + 4ull * blk);
 }
@@ -1277,7 +1288,7 @@ __global__ void __launch_bounds__(SWEEP_THREADS, (SweepOccupancy<S, RESID, false
   if constexpr (GEOM) {
     // the geometry does not change between sweeps: its word is on its way (or here) when
     // the previous sweep ends, so the population loads do not wait for it
-    uint32_t lm = geometry_word(a, blk);
+    uint32_t lm = geometry_word(a, blk * SWEEP_THREADS + threadIdx.x);
     wait_for_previous_sweep(blk, lm);
     sweep_block<S, RESID, MODE, GEOM>(a, blk, lm);
   } else {
@@ -1770,8 +1781,13 @@ __global__ void __launch_bounds__(SWEEP_THREADS, (SweepOccupancy<S, RESID, true,
         __syncthreads();
       }
       if constexpr (MODE == STREAM_AB) {
-        if (sa.links || sa.forced) sweep_block<S, RESID, MODE, true>(sa, b - lat_begin, geometry_word(sa, b - lat_begin));
-        else sweep_block<S, RESID, MODE, false>(sa, b - lat_begin);
+        if (sa.links || sa.forced) {
+          const uint32_t blk = b - lat_begin;
+          sweep_block<S, RESID, MODE, true>(sa, blk, geometry_word(sa, blk * SWEEP_THREADS + threadIdx.x));
+        }
+        else {
+          sweep_block<S, RESID, MODE, false>(sa, b - lat_begin);
+        }
       } else {
         sweep_block<S, RESID, MODE, false>(sa, b - lat_begin);
       }
@@ -2010,6 +2026,10 @@ static inline uint32_t bounds_errors_impl() {
   }                                                                                                     \
   template <> cudaError_t launch_resident<S>(const SweepArgs& a, int steps, bool swapped, cudaStream_t s) { \
     return launch_resident_impl<S>(a, steps, swapped, s);                                               \
+  }                                                                                                     \
+  template <> cudaError_t launch_grid_steps<S>(const SweepArgs& a, int steps, uint32_t* arrivals,         \
+                                               cudaStream_t s) {                                        \
+    return launch_grid_steps_impl<S>(a, steps, arrivals, s);                                            \
   }                                                                                                     \
   template <> cudaError_t launch_init<S>(void* dst, uint32_t N, double rho0, cudaStream_t s) {          \
     return launch_init_impl<S>(dst, N, rho0, s);                                                        \

@@ -172,7 +172,8 @@ struct SweepArgs {
 };
 
 // Error bits of SweepArgs::err.
-constexpr uint32_t ERR_STAGE_WAIT = 1u;
+constexpr uint32_t ERR_STAGE_WAIT = 1u;  // the row-staged sweep
+constexpr uint32_t ERR_GRID_WAIT = 2u;   // the grid barrier of the multi-step kernel
 
 // Geometry word of a node: bits 0..18 (nodes without a rule): the pull source of
 // population k is solid (mid-grid bounce-back); bits 24..29: the node's on-site rule
@@ -225,13 +226,19 @@ inline uint32_t partial_rows(uint32_t nblocks) { return nblocks + fold_groups(nb
 // loading and storing the state costs as much as the launches).
 constexpr uint32_t RESIDENT_THREADS = 512;
 constexpr uint32_t RESIDENT_CTAS = 16;
-constexpr uint32_t RESIDENT_NODES = RESIDENT_THREADS * RESIDENT_CTAS;
+constexpr uint32_t RESIDENT_NODES = RESIDENT_THREADS * RESIDENT_CTAS, RESIDENT_NODES_F64 = RESIDENT_NODES / 2;
 constexpr int RESIDENT_MIN_STEPS = 16;
+// Nodes beyond which no A/B lattice takes its steps in one launch of a block per SM (the
+// launch itself knows the SMs).
+constexpr uint32_t GRID_STEPS_NODES = 262144;
 
 // mode: 0 A/B pull, 1 AA gather-scatter step, 2 AA in-place step (see kernels.cuh)
 template <typename S> cudaError_t launch_sweep(const SweepArgs& a, bool resid, int mode, cudaStream_t s);
 // `steps` steps of a small lattice in one launch (resident.cuh), from src to dst
 template <typename S> cudaError_t launch_resident(const SweepArgs& a, int steps, bool swapped, cudaStream_t s);
+// `steps` A/B steps of a lattice that one block per SM covers, in one launch; arrivals: a
+// device word for its grid barrier
+template <typename S> cudaError_t launch_grid_steps(const SweepArgs& a, int steps, uint32_t* arrivals, cudaStream_t s);
 template <typename S> cudaError_t launch_init(void* dst, uint32_t N, double rho0, cudaStream_t s);
 // swapped: the state holds f_k in slot -k (an AA lattice between step pairs)
 template <typename S> cudaError_t launch_macros(const void* src, uint32_t N, double rho0, void* rho,

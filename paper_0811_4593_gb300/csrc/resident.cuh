@@ -9,8 +9,10 @@
 // memory (their addresses are formed once), and a cluster barrier separates the steps.
 // The node code is the sweep's, so the bits are.
 //
-// A cluster has 16 SMs of the chip's 152, so the rule ends where their arithmetic takes
-// as long as the launches they replace: RESIDENT_NODES.
+// A cluster has 16 SMs of the chip's 152, so it ends where the whole chip between grid
+// barriers (below) is as fast: 8,192 nodes, FP64 4,096. Per step, cluster against grid:
+// FP32 periodic 8,192 nodes 1.5 against 2.0 us; FP64 4,096 nodes 2.9 against 3.1, 8,192
+// nodes 5.1 against 3.2.
 #pragma once
 
 namespace lbm {
@@ -153,6 +155,103 @@ template <typename S>
 cudaError_t launch_resident_impl(const SweepArgs& a, int steps, bool swapped, cudaStream_t s) {
   if (a.links || a.forced) return launch_resident_geom<S, true>(a, steps, swapped, s);
   return launch_resident_geom<S, false>(a, steps, swapped, s);
+}
+
+// ---------------------------------------------------------------------------------
+// Many steps of a lattice that one block per SM covers, in one launch: each thread keeps
+// its node, the arrays stay in global memory (L2), and a grid barrier separates the steps.
+// A launch per step of such a lattice pays for the launch, for the fetch of its
+// instructions into every SM's cache and for the drain of the wave; the barrier is one
+// atomic per block and a poll through L2. The node code is the sweep's. One block per SM
+// and no more, so that few arrive at the barrier (with 256-node blocks, several per SM, a
+// step of 64 x 64 x 32 FP32 took 4.8 us, with one block 3.7, by launches 5.0).
+// ---------------------------------------------------------------------------------
+
+// Nodes a block holds at most, and so the largest lattice (152 SMs: 155,648 nodes, FP64
+// 77,824): the threads that its registers allow without spills. Beyond, launches are as
+// fast: 64 x 64 x 32 FP32 with a body force 5.4 against 5.6 us, 99 x 33 x 33 FP64 (with
+// 768 threads and spills) 10.2 against 9.3 us.
+template <typename S> constexpr int grid_step_threads() { return std::is_same<S, double>::value ? 512 : 1024; }
+
+// Grid barrier: every block arrives and waits for `target` arrivals; false once the wait
+// has taken STAGE_WAIT_LIMIT_NS (the blocks of a cooperative launch are all resident, so
+// it ends; the limit bounds it all the same). Every thread of the block takes part.
+__device__ __forceinline__ bool grid_barrier(uint32_t* arrivals, uint32_t target, const SweepArgs& a) {
+  __shared__ bool ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (!(a.drop_copies && blockIdx.x == 0))  // test hook: the wait runs out
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrivals) : "memory");
+    uint32_t seen;
+    uint64_t t0 = 0;
+    bool in_time = true;
+    for (uint32_t spins = 0;; ++spins) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(arrivals) : "memory");
+      if (seen >= target) break;
+      if ((spins & 1023u) == 1023u) {
+        const uint64_t now = global_ns();
+        if (t0 == 0) t0 = now;
+        else if (now - t0 > STAGE_WAIT_LIMIT_NS) {
+          if (a.err) atomicOr(a.err, ERR_GRID_WAIT);
+          in_time = false;
+          break;
+        }
+      }
+    }
+    ok = in_time;
+  }
+  __syncthreads();
+  return ok;
+}
+
+// `a` goes from array 0 to array 1, `b` back.
+template <typename S, bool GEOM>
+__global__ void __launch_bounds__((grid_step_threads<S>()), 1)
+    grid_steps_kernel(const __grid_constant__ SweepArgs a, const __grid_constant__ SweepArgs b, int steps,
+                      uint32_t* arrivals) {
+  const uint32_t cell = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t lm = GEOM ? geometry_word(a, cell) : 0u;
+  NodeTerms<typename ComputeOf<S>::T> unused;
+  for (int s = 0;;) {
+    sweep_node<S, false, STREAM_AB, GEOM, true>((s & 1) ? b : a, cell, lm, unused);
+    if (++s == steps) break;
+    if (!grid_barrier(arrivals, uint32_t(s) * gridDim.x, a)) break;
+  }
+}
+
+template <typename S, bool GEOM>
+cudaError_t launch_grid_steps_geom(const SweepArgs& a, int steps, uint32_t* arrivals, cudaStream_t s) {
+  const void* fn = reinterpret_cast<const void*>(grid_steps_kernel<S, GEOM>);
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const uint32_t per = ((a.N + uint32_t(sms) - 1) / uint32_t(sms) + 31u) / 32u * 32u;
+  const uint32_t blocks = (a.N + per - 1) / per;
+  if (per > uint32_t(grid_step_threads<S>()) || uint64_t(steps) * blocks >= (1ull << 32)) return cudaErrorNotSupported;
+  e = cudaMemsetAsync(arrivals, 0, sizeof(uint32_t), s);
+  if (e != cudaSuccess) return e;
+  SweepArgs b = a;
+  b.src = a.dst;
+  b.dst = const_cast<void*>(a.src);
+  for (int k = 0; k < Q; ++k) {
+    b.src_pop[k] = a.dst_pop[k];
+    b.dst_pop[k] = const_cast<void*>(a.src_pop[k]);
+  }
+  SweepArgs first = a;
+  void* args[] = {&first, &b, &steps, &arrivals};
+  e = cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(per), args, 0, s);
+  if (e != cudaErrorCooperativeLaunchTooLarge) return e;
+  cudaGetLastError();  // fewer SMs are free for this process than the device has
+  return cudaErrorNotSupported;
+}
+
+// `steps` steps from src, alternating the two arrays; cudaErrorNotSupported where one block
+// per SM does not cover the lattice. `arrivals`: a device word of the caller's.
+template <typename S>
+cudaError_t launch_grid_steps_impl(const SweepArgs& a, int steps, uint32_t* arrivals, cudaStream_t s) {
+  if (a.links || a.forced) return launch_grid_steps_geom<S, true>(a, steps, arrivals, s);
+  return launch_grid_steps_geom<S, false>(a, steps, arrivals, s);
 }
 
 }  // namespace lbm

@@ -51,6 +51,7 @@ struct lbm_ctx {
   double* dred = nullptr;    // reduction results [4], and behind them
   uint32_t* derr = nullptr;  // the error word of the sweeps (SweepArgs::err)
   uint32_t* dticket = nullptr;  // and the fold's ticket
+  uint32_t* darrivals = nullptr;  // and the arrivals of the multi-step kernel's grid barrier
   cudaStream_t stream = nullptr;
   int64_t steps = 0, launches = 0, device_bytes = 0;
   std::string err = "no error";
@@ -296,12 +297,21 @@ cudaError_t dispatch_resident(lbm_ctx* ctx, int n) {
   }
 }
 
+cudaError_t dispatch_grid_steps(lbm_ctx* ctx, int n) {
+  switch (ctx->prec) {
+    case LBM_F64: return lbm::launch_grid_steps<double>(ctx->args, n, ctx->darrivals, ctx->stream);
+    case LBM_F32: return lbm::launch_grid_steps<float>(ctx->args, n, ctx->darrivals, ctx->stream);
+    default: return lbm::launch_grid_steps<__half>(ctx->args, n, ctx->darrivals, ctx->stream);
+  }
+}
+
 // Issues n plain steps: one launch each, or for a small lattice all of them (an even
 // number for AA, whose state it reads and leaves between step pairs) in one.
 lbm_status issue_steps(lbm_ctx* ctx, int n) {
   const bool aa = ctx->scheme == LBM_SCHEME_AA;
   const int m = aa ? n & ~1 : n;
-  if (ctx->N <= lbm::RESIDENT_NODES && m >= lbm::RESIDENT_MIN_STEPS && !(aa && ctx->steps % 2 != 0)) {
+  const uint32_t resident = ctx->prec == LBM_F64 ? lbm::RESIDENT_NODES_F64 : lbm::RESIDENT_NODES;
+  if (ctx->N <= resident && m >= lbm::RESIDENT_MIN_STEPS && !(aa && ctx->steps % 2 != 0)) {
     // m steps leave the state where m launches would: in the other array when m is odd
     set_direction(ctx, ctx->cur);
     if (m % 2 == 0) {
@@ -314,6 +324,17 @@ lbm_status issue_steps(lbm_ctx* ctx, int n) {
       ctx->steps += m;
       ctx->launches += 1;
       n -= m;
+    } else if (e != cudaErrorNotSupported) {
+      return cuda_fail(ctx, e, "multi-step launch");
+    }
+  } else if (!aa && ctx->N <= lbm::GRID_STEPS_NODES && n >= lbm::RESIDENT_MIN_STEPS) {
+    set_direction(ctx, ctx->cur);
+    const cudaError_t e = dispatch_grid_steps(ctx, n);
+    if (e == cudaSuccess) {
+      ctx->cur ^= n & 1;
+      ctx->steps += n;
+      ctx->launches += 1;
+      n = 0;
     } else if (e != cudaErrorNotSupported) {
       return cuda_fail(ctx, e, "multi-step launch");
     }
@@ -373,7 +394,10 @@ lbm_status report_device_error(lbm_ctx* ctx, uint32_t v) {
   if (v == 0) return LBM_OK;
   LBM_CUDA(ctx, cudaMemsetAsync(ctx->derr, 0, sizeof v, ctx->stream), "clearing the error word");
   return fail(ctx, LBM_ERR_CUDA,
-              "a sweep gave up waiting for its staged row copies (device error word 0x%x): the state is not valid", v);
+              v & lbm::ERR_STAGE_WAIT
+                  ? "a sweep gave up waiting for its staged row copies (device error word 0x%x): the state is not valid"
+                  : "a sweep gave up waiting for its other blocks (device error word 0x%x): the state is not valid",
+              v);
 }
 
 // Synchronises the stream, then reads (and clears) the sweeps' device error word.
@@ -466,11 +490,12 @@ lbm_status lbm_create_scheme(int nx, int ny, int nz, double tau, const lbm_face_
     if (!ctx->buf[b]) return bail(fail(ctx, LBM_ERR_OOM, "allocation of %zu bytes for populations failed", pop_bytes));
   }
   if (scheme == LBM_SCHEME_AA) ctx->buf[1] = ctx->buf[0];
-  const size_t red_bytes = 4 * sizeof(double) + 2 * sizeof(uint32_t);
+  const size_t red_bytes = 4 * sizeof(double) + 3 * sizeof(uint32_t);
   ctx->dred = static_cast<double*>(ctx_alloc(ctx, red_bytes));
   if (!ctx->dred) return bail(fail(ctx, LBM_ERR_OOM, "allocation of the reduction result failed"));
   ctx->derr = reinterpret_cast<uint32_t*>(ctx->dred + 4);
   ctx->dticket = ctx->derr + 1;
+  ctx->darrivals = ctx->derr + 2;
   e = cudaMemsetAsync(ctx->dred, 0, red_bytes, ctx->stream);
   if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "clearing the reduction result and the error word"));
 
