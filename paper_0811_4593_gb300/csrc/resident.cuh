@@ -45,38 +45,115 @@ __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
-// `per`: nodes per CTA (the block's threads). SWAPPED state (an AA lattice between step
-// pairs): population k lies in slot -k of the global array, at both ends. The new state
-// goes to dst.
+// Box boundary code of a node: fx + 3 fy + 9 fz as apply_boundary takes it.
+__device__ __forceinline__ int boundary_code(const SweepArgs& a, uint32_t x, uint32_t y, uint32_t z) {
+  const bool px = a.periodic & 1u, py = a.periodic & 2u, pz = a.periodic & 4u;
+  const int fx = px ? 0 : (x == 0 ? 1 : (x == a.nx - 1 ? 2 : 0));
+  const int fy = py ? 0 : (y == 0 ? 1 : (y == a.ny - 1 ? 2 : 0));
+  const int fz = pz ? 0 : (z == 0 ? 1 : (z == a.nz - 1 ? 2 : 0));
+  return fx + 3 * fy + 9 * fz;
+}
+
+// Which of a CTA's nodes each of its threads takes (NO_NODE: none). Either in node order,
+// or nodes of one closure side by side (each in node order), a new warp for each group
+// where the block has the threads. The slowest warp sets the pace of every step, and in
+// node order the warps at the ends of a narrow channel run the bodies of an x face, a z
+// face and two edges one after the other (4 x 4 x 256 FP32: 1.73 us per step, grouped 1.2).
+// Grouped, that is, where some warp has two closures to run, or where fewer closures are
+// run without more warps -- unless nx is a multiple of 8: the nodes of an x face then lie
+// in the same few banks, which costs more (16 x 16 x 16 FP32 channel: 1.64 against 1.40 us;
+// a gap word every 32 spreads them but slows all others). `key`: the group of the thread's
+// own node (0: no closure).
+constexpr uint32_t NODE_GROUPS = 28, NO_NODE = 0xffffu;
+__device__ __forceinline__ uint32_t grouped_node(uint32_t key, uint32_t nx) {
+  constexpr uint32_t WARPS = RESIDENT_THREADS / 32;
+  __shared__ uint32_t before[NODE_GROUPS][WARPS], start[NODE_GROUPS], count[NODE_GROUPS];
+  __shared__ uint32_t bodies[WARPS];
+  __shared__ uint16_t order[RESIDENT_THREADS];
+  __shared__ bool grouped;
+  const uint32_t tid = threadIdx.x, warp = tid >> 5;
+  const uint32_t same = __match_any_sync(0xffffffffu, key);
+  const uint32_t rank = __popc(same & ((1u << (tid & 31u)) - 1u));
+  for (uint32_t i = tid; i < NODE_GROUPS * WARPS; i += blockDim.x) before[i / WARPS][i % WARPS] = 0;
+  order[tid] = NO_NODE;
+  const uint32_t own = __popc(__ballot_sync(0xffffffffu, rank == 0 && key != 0u && key != NO_NODE));
+  const bool used = __any_sync(0xffffffffu, key != NO_NODE);
+  if ((tid & 31u) == 0) bodies[warp] = used ? own + 0x10000u : 0u;  // and one warp
+  __syncthreads();
+  if (key != NO_NODE && rank == 0) before[key][warp] = __popc(same);
+  __syncthreads();
+  if (tid < NODE_GROUPS) {
+    uint32_t sum = 0;
+    for (uint32_t w = 0; w < WARPS; ++w) {
+      const uint32_t n = before[tid][w];
+      before[tid][w] = sum;
+      sum += n;
+    }
+    count[tid] = sum;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    uint32_t now = 0, most = 0, whole = 0, next = 0;
+    for (uint32_t w = 0; w < blockDim.x / 32u; ++w) {
+      now += bodies[w];
+      most = most > (bodies[w] & 0xffffu) ? most : bodies[w] & 0xffffu;
+    }
+    for (uint32_t g = 0; g < NODE_GROUPS; ++g) whole += (count[g] + 31u) / 32u;
+    const uint32_t closures = whole - (count[0] + 31u) / 32u;
+    grouped = most > 1u || ((nx & 7u) != 0 && closures < (now & 0xffffu) && whole <= now >> 16);
+    const uint32_t mask = whole * 32u <= blockDim.x ? 31u : 0u;
+    for (uint32_t g = 0; g < NODE_GROUPS; ++g) {
+      start[g] = next;
+      next += (count[g] + mask) & ~mask;
+    }
+  }
+  __syncthreads();
+  if (!grouped) return key != NO_NODE ? tid : NO_NODE;
+  if (key != NO_NODE) order[start[key] + before[key][warp] + rank] = uint16_t(tid);
+  __syncthreads();
+  return order[tid];
+}
+
+// `per`: nodes per CTA, at most the block's threads. SWAPPED state (an AA lattice between
+// step pairs): population k lies in slot -k of the global array, at both ends. The new
+// state goes to dst.
 template <typename S, bool GEOM>
 __global__ void __launch_bounds__(RESIDENT_THREADS, 1)
-    resident_kernel(const __grid_constant__ SweepArgs a, int steps, bool swapped) {
+    resident_kernel(const __grid_constant__ SweepArgs a, int steps, uint32_t per, bool swapped) {
   using T = typename ComputeOf<S>::T;
   extern __shared__ __align__(16) unsigned char resident_smem[];
   S* const buf = reinterpret_cast<S*>(resident_smem);  // [2][19][per]
-  const uint32_t per = blockDim.x, tid = threadIdx.x;
-  const uint32_t cell = blockIdx.x * per + tid;
-  uint32_t lm = 0;
-  if (GEOM && a.links && cell < a.N) lm = __ldg(a.links + cell);
-  // solid nodes keep their populations, in both global arrays, and nobody reads them
-  const bool active = cell < a.N && !(lm & SOLID_NODE);
-  const uint32_t array_bytes = Q * per * uint32_t(sizeof(S));
-  uint32_t from[Q];  // shared-window addresses of the pull sources in array 0
-  uint32_t x = 0, y = 0, z = 0;
-  int code = 0;
-  if (active) {
+  auto place = [&](uint32_t cell, uint32_t& x, uint32_t& y, uint32_t& z) {
     const uint32_t q1 = fdiv(a.div_nx, cell);
     x = cell - q1 * a.nx;
     z = fdiv(a.div_ny, q1);
     y = q1 - z * a.ny;
+  };
+  uint32_t x = 0, y = 0, z = 0, key = NO_NODE, lm = 0;
+  uint32_t cell = blockIdx.x * per + threadIdx.x;
+  if (threadIdx.x < per && cell < a.N) {
+    place(cell, x, y, z);
+    if (GEOM) lm = geometry_word(a, cell);
+    const uint32_t c = uint32_t(boundary_code(a, x, y, z));
+    // both x faces share a body; solid nodes keep their populations, in both global
+    // arrays, and nobody reads them
+    key = ((lm >> RULE_SHIFT) & RULE_BITS) ? NODE_GROUPS - 1 : (c == 2u ? 1u : c);
+    if (lm & SOLID_NODE) key = NO_NODE;
+  }
+  const uint32_t node = grouped_node(key, a.nx);
+  const bool active = node != NO_NODE;
+  const uint32_t array_bytes = Q * per * uint32_t(sizeof(S));
+  uint32_t from[Q];  // shared-window addresses of the pull sources in array 0
+  int code = 0;
+  if (active) {
+    cell = blockIdx.x * per + node;
+    place(cell, x, y, z);
+    lm = GEOM ? geometry_word(a, cell) : 0u;
+    code = boundary_code(a, x, y, z);
     const bool px = a.periodic & 1u, py = a.periodic & 2u, pz = a.periodic & 4u;
     const uint32_t xm = x ? x - 1 : (px ? a.nx - 1 : 0), xp = (x + 1 < a.nx) ? x + 1 : (px ? 0 : a.nx - 1);
     const uint32_t ym = y ? y - 1 : (py ? a.ny - 1 : 0), yp = (y + 1 < a.ny) ? y + 1 : (py ? 0 : a.ny - 1);
     const uint32_t zm = z ? z - 1 : (pz ? a.nz - 1 : 0), zp = (z + 1 < a.nz) ? z + 1 : (pz ? 0 : a.nz - 1);
-    const int fx = px ? 0 : (x == 0 ? 1 : (x == a.nx - 1 ? 2 : 0));
-    const int fy = py ? 0 : (y == 0 ? 1 : (y == a.ny - 1 ? 2 : 0));
-    const int fz = pz ? 0 : (z == 0 ? 1 : (z == a.nz - 1 ? 2 : 0));
-    code = fx + 3 * fy + 9 * fz;
     const bool links = GEOM && (lm & ~(RULE_BITS << RULE_SHIFT)) != 0u;
     static_for<0, Q>([&](auto kc) {
       constexpr int k = decltype(kc)::value;
@@ -89,7 +166,7 @@ __global__ void __launch_bounds__(RESIDENT_THREADS, 1)
       const uint32_t rank = source / per;
       from[k] = cluster_address(smem_u32(buf + slot * per + (source - rank * per)), rank);
       const S* own = static_cast<const S*>(a.src_pop[swapped ? opp(k) : k]);
-      buf[k * per + tid] = own[cell];
+      buf[k * per + node] = own[cell];
     });
   }
   cluster_barrier();
@@ -109,7 +186,7 @@ __global__ void __launch_bounds__(RESIDENT_THREADS, 1)
           static_cast<S*>(a.dst_pop[swapped ? opp(k) : k])[cell] = Storage<S>::store(h[k]);
         });
       } else {
-        S* to = buf + ((s & 1) ? 0u : Q * per) + tid;
+        S* to = buf + ((s & 1) ? 0u : Q * per) + node;
         static_for<0, Q>([&](auto kc) { to[decltype(kc)::value * per] = Storage<S>::store(h[decltype(kc)::value]); });
       }
     }
@@ -124,13 +201,18 @@ cudaError_t launch_resident_geom(const SweepArgs& a, int steps, bool swapped, cu
   // as many CTAs as a cluster has, whole warps each
   const uint32_t per = ((a.N + RESIDENT_CTAS - 1) / RESIDENT_CTAS + 31u) / 32u * 32u;
   const uint32_t ctas = (a.N + per - 1) / per;
+  // more warps than the nodes fill, so that the groups of grouped_node can start at warp
+  // boundaries: eight, or for FP64, whose steps are bound by the warps on a scheduler, no
+  // more than fill up a set of four
+  const uint32_t more = std::is_same<S, double>::value ? (per + 127u) / 128u * 128u : per + 256u;
+  const uint32_t threads = more < RESIDENT_THREADS ? more : RESIDENT_THREADS;
   const size_t smem = size_t(2) * Q * per * sizeof(S);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctas);
-  cfg.blockDim = dim3(per);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -146,7 +228,7 @@ cudaError_t launch_resident_geom(const SweepArgs& a, int steps, bool swapped, cu
     cudaGetLastError();
     return cudaErrorNotSupported;
   }
-  return cudaLaunchKernelEx(&cfg, resident_kernel<S, GEOM>, a, steps, swapped);
+  return cudaLaunchKernelEx(&cfg, resident_kernel<S, GEOM>, a, steps, per, swapped);
 }
 
 // `steps` steps from src to dst (which may be the same array); cudaErrorNotSupported where
