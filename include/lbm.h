@@ -184,7 +184,9 @@ LBM_API lbm_status lbm_get_populations(lbm_ctx* ctx, void* dst, int z0, int nzs,
  * (copied, not retained). Fluid nodes next to a solid node take the mid-grid
  * bounce-back of Sec. "Boundary conditions" for the populations that would stream in
  * from it: f_i(x) = f*_-i(x), the population the node sent towards the wall, reversed.
- * Solid nodes keep their populations. Costs 4 bytes per node of extra traffic per step.
+ * Solid nodes keep their populations; plain steps neither read nor write them. Costs 4
+ * bytes per node of extra traffic per step, or where an eighth or more of the nodes are
+ * solid 8 bytes per fluid node (a list of them, 8 bytes per node of device memory).
  * A/B scheme only (LBM_ERR_ARG for AA). Synchronises. */
 LBM_API lbm_status lbm_set_solid(lbm_ctx* ctx, const uint8_t* solid);
 
@@ -214,7 +216,7 @@ LBM_API lbm_status lbm_set_solid(lbm_ctx* ctx, const uint8_t* solid);
  *                which keeps a resting node at rest).
  * A node with a code must be fluid, and every population it cannot stream (source solid,
  * or outside a walled axis) must be one its rule sets; otherwise LBM_ERR_ARG names the
- * node. Extra traffic: 4 bytes per node per step. A/B scheme only; not while the context
+ * node. Extra traffic and memory as for lbm_set_solid. A/B scheme only; not while the context
  * is attached to a batch (LBM_ERR_STATE). Synchronises. */
 LBM_API lbm_status lbm_set_geometry(lbm_ctx* ctx, const uint8_t* solid, const int8_t* code);
 

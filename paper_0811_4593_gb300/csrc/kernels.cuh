@@ -1153,6 +1153,14 @@ __device__ __forceinline__ uint32_t geometry_word(const SweepArgs& a, uint32_t c
   return a.links && cell < a.N ? __ldg(a.links + chk(cell, a.N)) : 0u;
 }
 
+// The i-th node that a plain step of a lattice with a geometry visits, and its geometry
+// word: from the list of fluid nodes where the lattice has one, else node i. Beyond the
+// last: a cell outside the lattice.
+__device__ __forceinline__ uint2 geometry_node(const SweepArgs& a, uint32_t i) {
+  if (!a.fluid) return make_uint2(i, geometry_word(a, i));
+  return i < a.nfluid ? __ldg(a.fluid + i) : make_uint2(~0u, 0u);
+}
+
 // ---------------------------------------------------------------------------------
 // The fused time step: pull stream, classify, close, collide, store.
 // ---------------------------------------------------------------------------------
@@ -1285,9 +1293,14 @@ template <typename S, bool RESID, int MODE, bool GEOM>
 __global__ void __launch_bounds__(SWEEP_THREADS, (SweepOccupancy<S, RESID, false, MODE, GEOM>::blocks))
     sweep_kernel(const __grid_constant__ SweepArgs a) {
   uint32_t blk = blockIdx.x;
-  if constexpr (GEOM) {
-    // the geometry does not change between sweeps: its word is on its way (or here) when
-    // the previous sweep ends, so the population loads do not wait for it
+  if constexpr (GEOM && !RESID) {
+    // the geometry does not change between sweeps: its words are on their way (or here)
+    // when the previous sweep ends, so the population loads do not wait for them
+    uint2 node = geometry_node(a, blk * SWEEP_THREADS + threadIdx.x);
+    wait_for_previous_sweep(node.x, node.y);
+    NodeTerms<typename ComputeOf<S>::T> unused;
+    sweep_node<S, false, MODE, true>(a, node.x, node.y, unused);
+  } else if constexpr (GEOM) {
     uint32_t lm = geometry_word(a, blk * SWEEP_THREADS + threadIdx.x);
     wait_for_previous_sweep(blk, lm);
     sweep_block<S, RESID, MODE, GEOM>(a, blk, lm);
@@ -1881,7 +1894,8 @@ inline cudaError_t launch_after(void (*kernel)(SweepArgs), uint32_t grid, uint32
 template <typename S, int MODE, bool GEOM>
 cudaError_t launch_sweep_mode(const SweepArgs& a, bool resid, cudaStream_t s) {
   auto kernel = resid ? sweep_kernel<S, true, MODE, GEOM> : sweep_kernel<S, false, MODE, GEOM>;
-  return launch_after(kernel, sweep_blocks(a.N), SWEEP_THREADS, 0, a, s);
+  const uint32_t nodes = GEOM && !resid ? plain_step_nodes(a) : a.N;
+  return launch_after(kernel, sweep_blocks(nodes > 0 ? nodes : 1), SWEEP_THREADS, 0, a, s);
 }
 
 // Stages of the row-staged sweep's shared-memory ring.

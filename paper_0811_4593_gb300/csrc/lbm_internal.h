@@ -157,6 +157,10 @@ struct SweepArgs {
   void* snap;         // residual steps: [3][N] velocity snapshot in the compute type
   double* partials;   // residual steps: [blocks][4] per-block sums, then [groups][4] of the fold
   const uint32_t* links;  // optional [N] geometry words (nullptr: no geometry), see below
+  // optional list of the fluid nodes (cell, geometry word) in cell order: plain steps then
+  // visit them only, in warps without idle lanes
+  const uint2* fluid;
+  uint32_t nfluid;
   uint32_t forced;        // nonzero: a body force acts (eq. gravity)
   double force[3];        // F: momentum the collision adds per step
   double tforce[3];       // tau F: the equilibrium velocity shift times rho
@@ -231,6 +235,9 @@ constexpr int RESIDENT_MIN_STEPS = 16;
 // Nodes beyond which no A/B lattice takes its steps in one launch of a block per SM (the
 // launch itself knows the SMs).
 constexpr uint32_t GRID_STEPS_NODES = 262144;
+
+// Nodes a plain step visits.
+inline uint32_t plain_step_nodes(const SweepArgs& a) { return a.fluid ? a.nfluid : a.N; }
 
 // mode: 0 A/B pull, 1 AA gather-scatter step, 2 AA in-place step (see kernels.cuh)
 template <typename S> cudaError_t launch_sweep(const SweepArgs& a, bool resid, int mode, cudaStream_t s);

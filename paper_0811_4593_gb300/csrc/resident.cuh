@@ -291,8 +291,12 @@ template <typename S, bool GEOM>
 __global__ void __launch_bounds__((grid_step_threads<S>()), 1)
     grid_steps_kernel(const __grid_constant__ SweepArgs a, const __grid_constant__ SweepArgs b, int steps,
                       uint32_t* arrivals) {
-  const uint32_t cell = blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t lm = GEOM ? geometry_word(a, cell) : 0u;
+  uint32_t cell = blockIdx.x * blockDim.x + threadIdx.x, lm = 0;
+  if constexpr (GEOM) {
+    const uint2 node = geometry_node(a, cell);
+    cell = node.x;
+    lm = node.y;
+  }
   NodeTerms<typename ComputeOf<S>::T> unused;
   for (int s = 0;;) {
     sweep_node<S, false, STREAM_AB, GEOM, true>((s & 1) ? b : a, cell, lm, unused);
@@ -308,8 +312,10 @@ cudaError_t launch_grid_steps_geom(const SweepArgs& a, int steps, uint32_t* arri
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const uint32_t per = ((a.N + uint32_t(sms) - 1) / uint32_t(sms) + 31u) / 32u * 32u;
-  const uint32_t blocks = (a.N + per - 1) / per;
+  const uint32_t nodes = GEOM ? plain_step_nodes(a) : a.N;
+  const uint32_t per = ((nodes + uint32_t(sms) - 1) / uint32_t(sms) + 31u) / 32u * 32u;
+  if (per == 0) return cudaErrorNotSupported;
+  const uint32_t blocks = (nodes + per - 1) / per;
   if (per > uint32_t(grid_step_threads<S>()) || uint64_t(steps) * blocks >= (1ull << 32)) return cudaErrorNotSupported;
   e = cudaMemsetAsync(arrivals, 0, sizeof(uint32_t), s);
   if (e != cudaSuccess) return e;
