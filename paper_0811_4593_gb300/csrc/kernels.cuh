@@ -1272,17 +1272,23 @@ __device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk, ui
 // budget is 65536 / (256 * blocks)). The float sweeps are memory-bound and need many
 // warps in flight to hide DRAM latency: 6 blocks (<= 42 registers) for the plain step,
 // single-lattice or batched (the batched kernel at 4 blocks served 14 % fewer jobs per
-// second; its spills are in the geometry path, which serving lattices do not take); the
-// residual variant carries the reduction and gets 5. The FP64 sweeps are bound by the
-// FP64 pipe and get room for their double registers.
-// The AA gather-scatter step also keeps its push targets and takes 2 blocks fewer, the
-// AA in-place step one fewer.
-// The general-geometry variant (GEOM) carries the rule dispatch and the force and is
-// compiled for 4 blocks (2 for FP64).
+// second; its spills are in the geometry path, which serving lattices do not take; 7
+// blocks: 3.14 against 2.94 ms per 512^3 FP32 step, binary16 251 x 127 x 190 at 5, 6 and 7
+// blocks 100, 97.7 and 108 us); the residual variant carries the reduction and gets 5.
+// The AA gather-scatter step also keeps its push targets: 5 blocks, the AA in-place step 6
+// (301 x 199 x 255 FP32: 352 us per step, with 4 and 5 blocks 370, with 4 and 6 365), in
+// batches and binary16 one fewer each. The general-geometry variant (GEOM) carries the
+// rule dispatch and the force and is compiled for 4 blocks (128 x 16 x 256 tilted channel,
+// FP32, at 3, 4 and 5 blocks: 7.5, 7.3 and 7.4 us). FP64 sweeps hold 19 populations in
+// register pairs: 3 blocks of 80 registers (256 x 64 x 64 at 2, 3 and 4: 72.5, 63.5 and
+// 67.1 us), 2 for the variants with more to keep.
 template <typename S, bool RESID, bool BATCHED, int MODE, bool GEOM = false>
 struct SweepOccupancy {
   static constexpr int base = RESID ? 5 : 6;
-  static constexpr int blocks = GEOM ? 4 : (MODE == 1 ? (base > 4 ? 4 : base - 1) : (MODE == 2 ? (base > 5 ? 5 : base) : base));
+  static constexpr int aa = std::is_same<S, float>::value && !BATCHED ? 4 + MODE
+                            : MODE == 1                               ? 4
+                                                                      : 5;
+  static constexpr int blocks = GEOM ? 4 : (MODE == 0 ? base : aa);
 };
 template <bool RESID, bool BATCHED, int MODE, bool GEOM>
 struct SweepOccupancy<double, RESID, BATCHED, MODE, GEOM> {
