@@ -357,7 +357,7 @@ LBM_API const char* lbm_batch_last_error(const lbm_batch* b);
  *                     sum |u|^2, number of nodes with a non-finite or non-positive
  *                     density or a non-finite velocity}; the residual of lbm_residual is
  *                     sqrt(sums[1]) / sqrt(sums[2])
- *  cuda_stream        stream for the two kernel launches (NULL = legacy default stream)
+ *  cuda_stream        stream for the kernel launches (NULL = legacy default stream)
  * Limit: at most 16,777,216 nodes (256^3); larger lattices get LBM_ERR_ARG with a
  * message naming the limit. Asynchronous; nothing is allocated and nothing is freed.
  * The first call on a device looks up the static array's device address (with that

@@ -21,8 +21,7 @@ constexpr uint32_t kStaticBlocks = 65536;
 constexpr uint32_t kStaticRows = kStaticBlocks + kStaticBlocks / lbm::FOLD_ROWS;
 constexpr int kMaxDevices = 64;
 
-// the last double holds the fold's ticket (zero when the library is loaded, and again
-// after every fold)
+// the last double holds the fold's ticket
 __device__ __align__(256) double g_static_partials[4 * kStaticRows + 1];
 
 std::mutex g_setup_mu;
@@ -100,7 +99,10 @@ extern "C" LBM_API lbm_status lbm_reduce_state_static(const void* populations, i
       break;
   }
   cudaError_t e = cudaGetLastError();
+  // cleared by every call: calls that overlap give wrong sums (they share the array), but
+  // must not leave a ticket behind that spoils later ones
   uint32_t* ticket = reinterpret_cast<uint32_t*>(partials + 4ull * kStaticRows);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ticket, 0, sizeof(uint32_t), s);
   if (e == cudaSuccess) e = lbm::launch_final_reduce(partials, blocks, sums, ticket, s);
   if (e != cudaSuccess) {
     char buf[256];
