@@ -302,7 +302,7 @@ void set_in_place(lbm_ctx* ctx) {
 
 // Whether pairs of steps of an A/B lattice run in place: where one of its arrays lies in L2
 // but the two do not. FP32, per step, A/B against in place on a 129 MB L2 (256 x 64 rows
-// and odd ones): 45 MB arrays 11.7 / 12.1 us, 60 MB 17.3 / 15.3, 80 MB 24.6 / 20.9, 100 MB
+// and odd ones): 45 MB arrays 11.7 / 12.1 us, 60 MB 17.3 / 15.3, 80 MB 24.6 / 20.4, 100 MB
 // 30.9 / 29.6, 118 MB 36.4 / 38.6. Binary16 (half the bytes for the same arithmetic) and
 // FP64 lattices were faster with two arrays at every size.
 bool in_place_pays(const lbm_ctx* ctx) {
@@ -694,15 +694,19 @@ static lbm_status copy_populations(lbm_ctx* ctx, void* host_or_dev, int z0, int 
   char* user = static_cast<char*>(host_or_dev);
   cudaMemcpyKind kind = to_ctx ? (where == LBM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice)
                                : (where == LBM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice);
-  for (int k = 0; k < 19; ++k) {
+  // the whole of an A/B state lies in the array as it does in the caller's buffer: one copy
+  // in place of 19 (about 2 us of host time each)
+  const bool whole = nzs == ctx->nz && ctx->scheme == LBM_SCHEME_AB;
+  const size_t bytes = whole ? 19 * slab : slab;
+  for (int k = 0; k < (whole ? 1 : 19); ++k) {
     // an AA lattice keeps population k in slot -k between step pairs
     const int slot = ctx->scheme == LBM_SCHEME_AA ? lbm::opp(k) : k;
     char* l = lat + (size_t(slot) * ctx->N + size_t(z0) * plane) * es;
     char* u = user + size_t(k) * slab;
-    LBM_CUDA(ctx, cudaMemcpyAsync(to_ctx ? l : u, to_ctx ? u : l, slab, kind, ctx->stream), "population copy");
+    LBM_CUDA(ctx, cudaMemcpyAsync(to_ctx ? l : u, to_ctx ? u : l, bytes, kind, ctx->stream), "population copy");
     // plain steps leave solid nodes alone in both arrays: the other one takes them too
     if (to_ctx && ctx->args.links)
-      LBM_CUDA(ctx, cudaMemcpyAsync(static_cast<char*>(ctx->buf[ctx->cur ^ 1]) + (l - lat), l, slab,
+      LBM_CUDA(ctx, cudaMemcpyAsync(static_cast<char*>(ctx->buf[ctx->cur ^ 1]) + (l - lat), l, bytes,
                                     cudaMemcpyDeviceToDevice, ctx->stream), "population copy");
   }
   LBM_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "synchronising the population copy");
