@@ -160,8 +160,11 @@ __host__ __device__ __forceinline__ void fixed_to_double(const FixedSums& q, con
 //   diagonals of the x-y plane (b = o + q_x + q_y, c = a_x v_y):
 //     (+,+) (b + a_x) + (2 c + a_y)      (+,-) (b + a_x) - (2 c + a_y)
 //     (-,-) (b - a_x) + (2 c - a_y)      (-,+) (b - a_x) - (2 c - a_y)
-// added to (1 - omega) f; the same relaxation as `collide` writes for double.
-__host__ __device__ __forceinline__ void fixed_relax(const int64_t (&f)[19], const FixedSums& q, const FixedArgs& fx,
+// added to (1 - omega) f; the same relaxation as `collide` writes for double. KEEP false:
+// omega = 1 (tau = 1, where a step replaces the populations by their equilibrium), without
+// the 19 products with zero, 9 % of a node's instructions; the bits are the same.
+template <bool KEEP>
+__host__ __device__ __forceinline__ void fixed_relax_to(const int64_t (&f)[19], const FixedSums& q, const FixedArgs& fx,
                                                      double (&h)[19]) {
   const Limbs y = limbs_of(fixed_three_halves_over(q.r));
   const Limbs w3 = limbs_of(fx.w3), keep = limbs_of(fx.keep);
@@ -176,7 +179,7 @@ __host__ __device__ __forceinline__ void fixed_relax(const int64_t (&f)[19], con
   int32_t least = INT32_MAX;
   int64_t v[19];
   auto set = [&](int k, int64_t eq) {
-    v[k] = mul63(f[k], keep) + eq;
+    v[k] = KEEP ? mul63(f[k], keep) + eq : eq;
     const int32_t top = int32_t(v[k] >> 32);
     least = top < least ? top : least;
   };
@@ -209,6 +212,12 @@ __host__ __device__ __forceinline__ void fixed_relax(const int64_t (&f)[19], con
 #pragma unroll
     for (int k = 0; k < 19; ++k) h[k] = double(v[k]) * fx.unit_out;
   }
+}
+
+__host__ __device__ __forceinline__ void fixed_relax(const int64_t (&f)[19], const FixedSums& q, const FixedArgs& fx,
+                                                     double (&h)[19]) {
+  if ((fx.keep[0] | fx.keep[1]) == 0) fixed_relax_to<false>(f, q, fx, h);
+  else fixed_relax_to<true>(f, q, fx, h);
 }
 
 }  // namespace lbm

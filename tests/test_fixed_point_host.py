@@ -90,6 +90,12 @@ int main() {
             s.y += fx.force[1];
             s.z += fx.force[2];
             fixed_relax(f, s, fx, g);
+            if (tau == 1.0) {  // the products with zero left out
+              double t[19];
+              fixed_relax_to<true>(f, s, fx, t);
+              for (int k = 0; k < 19; ++k)
+                if (t[k] != g[k]) return fail("tau = 1", t[k], g[k]);
+            }
             for (int k = 0; k < 19; ++k) {
               const double e = double(std::fabs(R(g[k]) - q[k])) / rho0, ed = double(std::fabs(R(d[k]) - q[k])) / rho0;
               worst = e > worst ? e : worst;
