@@ -107,10 +107,11 @@ def code_only(text: str) -> str:
 
 
 def sweep_source_hash() -> str:
-    """Hash of the sweep's code (kernels.cuh, d3q19.cuh; comments excluded): a profiled
-    traffic figure is reported only while this matches the hash it was captured on."""
+    """Hash of the sweep's code (kernels.cuh, d3q19.cuh, fixed64.cuh, fixed_close.cuh;
+    comments excluded): a profiled traffic figure is reported only while this matches the
+    hash it was captured on."""
     h = hashlib.sha256()
-    for f in ("kernels.cuh", "d3q19.cuh"):
+    for f in ("kernels.cuh", "d3q19.cuh", "fixed64.cuh", "fixed_close.cuh"):
         with open(os.path.join(ROOT, "paper_0811_4593_gb300", "csrc", f), encoding="utf-8") as fh:
             h.update(code_only(fh.read()).encode())
     return h.hexdigest()[:16]
@@ -270,22 +271,6 @@ def whole_job_mlups(world: int, nodes: int, steps: int, max_ms: float) -> float:
     return world * nodes * steps / (max_ms * 1e-3) / 1e6
 
 
-# GB300's FP64 pipe: NVIDIA's 1.25 TFLOP/s FP64 figure is 2 DFMA per SM per clock at
-# 152 SMs and 2.07 GHz, i.e. 2 FP64 instructions per SM per clock.
-FP64_INST_PER_SM_CLOCK = 2.0
-
-
-def profiled_fp64_per_node(wl_name: str):
-    """FP64 instructions per node update of the FP64 sweep from the committed ncu
-    counters, if they were taken on the current sweep source."""
-    try:
-        with open(os.path.join(ROOT, "profiles", "traffic.json")) as fh:
-            rec = json.load(fh)[f"sweep/f64/{wl_name}"]
-    except Exception:  # noqa: BLE001
-        return None
-    return rec.get("fp64_inst_per_node") if rec.get("source_sha") == sweep_source_hash() else None
-
-
 def sweep_kernel_name(wl, precision, scheme="ab"):
     """The kernel that runs the plain (non-residual) steps of a lattice."""
     if precision == "f16" and wl.nx % 2 == 0 and getattr(wl, "solid", None) is None \
@@ -309,29 +294,6 @@ def run_variant(wl, precision, steps, warmup, resid_every, dist_ctx, clocks=None
            "bytes_per_update": BYTES_PER_UPDATE[precision], "scheme": scheme,
            "kernel": sweep_kernel_name(wl, precision, scheme),
            "resident_bytes_per_node": BYTES_PER_UPDATE[precision] // (2 if scheme == "aa" else 1)}
-    if precision == "f64":
-        # the FP64 sweep is bound by the FP64 pipe, not by HBM: its peak is the measured
-        # FP64 FMA rate of this device (thread-level operations per second; FP64 adds and
-        # multiplies issue at the same rate), the spec-derived figure is context only
-        from paper_0811_4593_gb300._binding import fp64_fma_rate
-        sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
-        mhz = (clocks or {}).get("sm_mhz") or 2070.0
-        nominal = FP64_INST_PER_SM_CLOCK * sms * mhz * 1e6 / 1e9
-        clk = ClockSampler(torch.cuda.current_device()).start()
-        rate, probe_ms = fp64_fma_rate(12000)
-        probe_clock = clk.stop()
-        peak = rate / 1e9
-        per_node = profiled_fp64_per_node("channel256")
-        alu = {"bound": "alu", "unit": "G FP64 inst/s", "peak": round(peak, 1), "peak_source": "measured",
-               "peak_basis": (f"lbm_fp64_fma_rate: 8 independent DFMA chains per thread on every resident warp, "
-                              f"{probe_ms:.1f} ms, SM clock {probe_clock.get('sm_mhz')} MHz"),
-               "nominal": round(nominal, 1),
-               "nominal_basis": f"{FP64_INST_PER_SM_CLOCK:g} FP64 inst / SM / clock x {sms} SMs x {mhz:g} MHz",
-               "fp64_inst_per_node": per_node}
-        if per_node:
-            a = per_node * wl.cells / (step_ms * 1e-3) / 1e9
-            alu.update(achieved=round(a, 1), frac=round(a / peak, 4))
-        out["roofline"] = alu
     return out
 
 

@@ -50,11 +50,13 @@ typedef enum {
 } lbm_status;
 
 /* Storage of the populations and the arithmetic of the sweep.
- *  LBM_F64          f_i stored as double; all arithmetic in double.
+ *  LBM_F64          f_i stored as double; arithmetic in 64-bit fixed point, at least as
+ *                   exact as in double, on nodes whose populations lie near a flow's
+ *                   (see fixed64.cuh), in double on any other; reductions in double.
  *  LBM_F32          shifted populations h_i = f_i - w_i rho0 stored as float;
  *                   arithmetic in float except the density of a face closure (eq. uin
- *                   and its appendix analogues), which is formed in double, and the
- *                   reductions, which accumulate in double.
+ *                   and its appendix analogues), which is formed as a float pair,
+ *                   and the reductions, which accumulate as float pairs and in double.
  *  LBM_F16_SHIFTED  h_i = f_i - w_i rho0 stored as IEEE binary16 (round to nearest
  *                   even); arithmetic as for LBM_F32. */
 typedef enum { LBM_F64 = 0, LBM_F32 = 1, LBM_F16_SHIFTED = 2 } lbm_precision;
@@ -375,8 +377,7 @@ LBM_API lbm_status lbm_reduce_state_static(const void* populations, int nx, int 
  * launch), timed with CUDA events on the legacy default stream. Writes thread-level
  * DFMA operations per second to *fma_per_s and the timed launch's duration in
  * milliseconds to *ms (may be NULL). Synchronises. LBM_ERR_ARG for iters < 1 or a NULL
- * fma_per_s; LBM_ERR_CUDA if a launch fails. The FP64 sweep's roofline divides its
- * FP64 instruction rate by this rate. */
+ * fma_per_s; LBM_ERR_CUDA if a launch fails. What arithmetic in double would be held to. */
 LBM_API lbm_status lbm_fp64_fma_rate(int iters, double* fma_per_s, double* ms);
 
 /* Last error message of a context, or of the calling thread's last failed call that

@@ -6,8 +6,8 @@
 // deviation from rest rather than to f_i. The closure and collision rules hold
 // unchanged for h (sum_i w_i c_i = 0, and the weights of the density relation sum to
 // one), with every density written as rho0 + (sum of h). FP64 storage holds f_i itself;
-// the same code runs on it with the reference density 0 (then "sum of h" is rho), which
-// spares the FP64 pipe the 38 shift additions per node.
+// the same code runs on it with the reference density 0 (then "sum of h" is rho). Most FP64
+// nodes take neither closure nor collision here but in fixed point (fixed64.cuh).
 #pragma once
 #include <cuda_fp16.h>
 #include <type_traits>
@@ -803,7 +803,7 @@ __device__ __forceinline__ Moments<float> moments_compensated(const float (&h)[Q
 //   a_i = 3 c_i.j
 // (j = rho u), which equals w_i (drho + rho (3 c.u + 9/2 (c.u)^2 - 3/2 u^2)) (eq. feq)
 // term by term and shares the symmetric part between the two populations. omega w_i is
-// folded into the per-class factors. The FP64 sweep, bound by the FP64 pipe, writes the
+// folded into the per-class factors. FP64 (the nodes outside fixed point) writes the
 // quadratic term as the momentum term A_i = 3 omega w_i (c_i.j) times c_i.u' with
 // u' = 3/2 u (omega w_i s_i = A_i (c_i.u'), b = drho - j.u'), one multiply fewer per
 // pair; the float sweeps, bound by memory, keep g_i (c_i.j)(c_i.u) with
@@ -1106,8 +1106,8 @@ __device__ __forceinline__ void relax_node(const SweepArgs& a, T (&h)[Q], uint32
   if (!solid) collide<std::is_same<S, float>::value>(h, m, omega_of<T>(a), a.mom_coef);
 }
 
-// Closure and relaxation of an FP64 node in fixed point; false, with h unchanged in no
-// particular way, where the node has to be taken in double.
+// Closure and relaxation of an FP64 node in fixed point; false, with h in no particular
+// state, where the node has to be taken in double.
 template <bool RESID, bool GEOM>
 __device__ __forceinline__ bool update_fixed(const SweepArgs& a, uint32_t lm, int code, uint32_t x, uint32_t y, uint32_t z,
                                              uint32_t cell, double (&h)[Q], NodeTerms<double>& terms) {

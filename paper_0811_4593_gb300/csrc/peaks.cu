@@ -1,6 +1,6 @@
 // peaks.cu -- measurement helper: the device's FP64 fused multiply-add rate.
 //
-// The FP64 sweep is bound by the FP64 pipe, so its roofline is the rate at which the
+// What FP64 arithmetic would be held to (the sweeps' was, before it moved to fixed point): the rate at which the
 // device retires double-precision FMAs. The kernel keeps every resident warp busy with
 // eight independent FMA chains per thread (enough to cover the pipe's latency) and is
 // timed with CUDA events; the result is thread-level DFMA operations per second.
