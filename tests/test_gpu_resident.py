@@ -82,3 +82,31 @@ def test_a_grid_barrier_that_runs_out_is_reported_and_the_context_recovers():
             l.set_populations(s0)
             l.step(20)
         np.testing.assert_array_equal(lat.get_populations(), ref.get_populations())
+
+
+@pytest.mark.parametrize("wl,prec,n", [(inp.couette(), "f64", 20), (inp.couette(), "f32", 2),
+                                       (inp.channel(33, 20, 21, 0.8, (0.02, 0.01, 0.0)), "f32", 18),
+                                       (inp.channel(256, 56, 56, 0.8, (0.02, 0.01, 0.0)), "f32", 4),
+                                       (inp.channel(256, 9, 7, 0.8, (0.02, 0.01, 0.0)), "f16", 4)],
+                         ids=["cluster", "launches", "grid", "in_place", "rows"])
+def test_captured_steps_replay(wl, prec, n):
+    # an even number of steps captured once and replayed: the state of as many steps
+    import torch
+
+    import paper_0811_4593_gb300 as lbm
+    s0 = encode(noisy_state((19, wl.nz, wl.ny, wl.nx), 6, amp=0.005), prec)
+    stream = torch.cuda.Stream()
+    with lbm.Lattice.from_workload(wl, prec, stream=stream) as lat, lbm.Lattice.from_workload(wl, prec) as ref:
+        for l in (lat, ref):
+            l.set_populations(s0)
+            l.step(n)
+        lat.sync()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            lat.step(n)
+        for _ in range(3):
+            graph.replay()
+        torch.cuda.synchronize()
+        for _ in range(3):
+            ref.step(n)
+        np.testing.assert_array_equal(lat.get_populations(), ref.get_populations())
