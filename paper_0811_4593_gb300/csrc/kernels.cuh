@@ -111,9 +111,10 @@ __device__ __forceinline__ uint32_t chk(uint32_t i, uint32_t) { return i; }
 // Programmatic dependent launch: consecutive sweeps of a stream are launched with the
 // serialisation relaxed (launch_after), so the next sweep's blocks are placed while the
 // last ones of this sweep run, and wait here, before their first access to memory, until
-// it has completed and its stores are visible. `index` ties every address to the wait:
-// loads written as plain functions of a pointer may otherwise be moved above it. Without
-// such a launch both instructions do nothing.
+// it has completed and its stores are visible to ordinary loads (not to non-coherent ones,
+// see load_pop). `index` ties every address to the wait: loads written as plain functions
+// of a pointer may otherwise be moved above it. Without such a launch both instructions do
+// nothing.
 // `ahead`: a value that no sweep writes, loaded before the wait.
 __device__ __forceinline__ void wait_for_previous_sweep(uint32_t& index, uint32_t& ahead) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -178,19 +179,18 @@ __host__ __device__ constexpr int first_nonzero(int a) {
 }
 
 // Storage codec: stored value <-> register value v (h_i for shifted storage, f_i for
-// FP64) in the compute type.
+// FP64) in the compute type. Its loads are read-only (non-coherent) ones: for the read-outs,
+// which are launched behind whatever wrote the array and write nothing into it. Sweeps load
+// through load_pop.
 template <typename S> struct Storage;
 template <> struct Storage<double> {
   static constexpr bool shifted = false;
   __device__ static double load(const double* p) { return __ldg(p); }
   __device__ static double store(double v) { return v; }
 };
-// FP32 loads are read-only loads that also ask L2 to fetch the enclosing 256-byte block
-// (PTX ld.global.nc with the .L2::256B prefetch-size qualifier): consecutive warps read
-// consecutive 128-byte pieces of each population row. Measured: the single-lattice
-// sweep unchanged, the batched sweep on a serving mix 1 - 2 % faster.
 template <> struct Storage<float> {
   static constexpr bool shifted = true;
+  // with the L2 prefetch hint of load_pop
   __device__ static float load(const float* p) {
     float v;
     asm("ld.global.nc.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
@@ -204,22 +204,30 @@ template <> struct Storage<__half> {
   __device__ static __half store(float v) { return __float2half_rn(v); }
 };
 
-// Population load of a sweep step: the A/B step reads through the storage codec (for
-// FP32 with the L2 prefetch hint); the AA steps read plain read-only loads (with the
-// hint the FP32 AA steps, which write the array they read, measured 2.6 % slower).
-template <typename S, int MODE>
+// Population load of a sweep step. An ordinary load, never a non-coherent one (ld.global.nc,
+// __ldg): those need data that nobody writes while the kernel lives, and the blocks of a
+// sweep are live while the sweep before it still stores the array they will read
+// (wait_for_previous_sweep); the AA steps write the array they read. What the wait makes
+// visible, it makes visible to ordinary loads. The A/B step of FP32 lattices also asks L2
+// for the enclosing 256-byte block (the .L2::256B prefetch-size qualifier): consecutive
+// warps read consecutive 128-byte pieces of each population row. Measured: the
+// single-lattice sweep unchanged, the batched sweep on a serving mix 1 - 2 % faster, the
+// AA steps 2.6 % slower, which go without.
+// COHERENT: written by other blocks of the same launch, so read through L2.
+template <typename S, int MODE, bool COHERENT = false>
 __device__ __forceinline__ typename std::conditional<std::is_same<S, double>::value, double, float>::type
 load_pop(const S* p) {
-  if constexpr (MODE != 0 && std::is_same<S, float>::value) return __ldg(p);
-  else return Storage<S>::load(p);
-}
-
-template <typename S, bool COHERENT>
-__device__ __forceinline__ typename std::conditional<std::is_same<S, double>::value, double, float>::type
-load_source(const S* p) {
-  if constexpr (!COHERENT) return Storage<S>::load(p);
-  else if constexpr (std::is_same<S, __half>::value) return __half2float(__ldcg(p));
-  else return __ldcg(p);
+  if constexpr (std::is_same<S, __half>::value) {
+    return __half2float(COHERENT ? __ldcg(p) : *p);
+  } else if constexpr (COHERENT) {
+    return __ldcg(p);
+  } else if constexpr (std::is_same<S, float>::value && MODE == 0) {
+    float v;
+    asm("ld.global.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+  } else {
+    return *p;
+  }
 }
 
 // The reference density the register values are shifted by: rho0, or 0 for FP64.
@@ -1211,7 +1219,7 @@ __device__ __forceinline__ void sweep_node(const SweepArgs& a, uint32_t cell, ui
         static_for<0, Q>([&](auto kc) {
           constexpr int k = decltype(kc)::value;
           if constexpr (MODE == STREAM_AB) {
-            h[k] = load_source<S, COHERENT>(static_cast<const S*>(a.src_pop[k]) + pull_idx(kc));
+            h[k] = load_pop<S, MODE, COHERENT>(static_cast<const S*>(a.src_pop[k]) + pull_idx(kc));
           } else if constexpr (MODE == STREAM_AA_GATHER) {
             h[k] = load_pop<S, MODE>(static_cast<const S*>(a.src_pop[opp(k)]) + pull_idx(kc));
           } else {
@@ -1229,7 +1237,7 @@ __device__ __forceinline__ void sweep_node(const SweepArgs& a, uint32_t cell, ui
           const S* p = own ? static_cast<const S*>(a.src_pop[k]) + cell
                            : (back ? static_cast<const S*>(a.src_pop[opp(k)]) + cell
                                    : static_cast<const S*>(a.src_pop[k]) + pull_idx(kc));
-          h[k] = load_source<S, COHERENT>(p);
+          h[k] = load_pop<S, MODE, COHERENT>(p);
         });
       }
     };
@@ -1326,18 +1334,18 @@ __global__ void __launch_bounds__(SWEEP_THREADS, (SweepOccupancy<S, RESID, false
 // stored as one half2. Each node runs the single-node sweep's closure,
 // moment and collision code, so both sweeps give the same bits.
 // ---------------------------------------------------------------------------------
-// Read-only loads that also ask L2 to fetch the enclosing 256-byte block (PTX
-// ld.global.nc with the .L2::256B prefetch-size qualifier): consecutive warps stream
+// Loads that also ask L2 to fetch the enclosing 256-byte block (the .L2::256B
+// prefetch-size qualifier; ordinary loads, see load_pop): consecutive warps stream
 // consecutive 128-byte pieces of each population row, so the next warp's data is
 // already on its way when it asks.
 __device__ __forceinline__ float ld_half_l2(const __half* p) {
   unsigned short v;
-  asm("ld.global.nc.L2::256B.u16 %0, [%1];" : "=h"(v) : "l"(p));
+  asm("ld.global.L2::256B.u16 %0, [%1];" : "=h"(v) : "l"(p));
   return __half2float(__ushort_as_half(v));
 }
 __device__ __forceinline__ void ld_half2_l2(const __half* p, float& lo, float& hi) {
   unsigned int v;
-  asm("ld.global.nc.L2::256B.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  asm("ld.global.L2::256B.u32 %0, [%1];" : "=r"(v) : "l"(p));
   lo = __half2float(__ushort_as_half(static_cast<unsigned short>(v & 0xffffu)));
   hi = __half2float(__ushort_as_half(static_cast<unsigned short>(v >> 16)));
 }
