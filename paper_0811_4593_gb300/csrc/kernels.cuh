@@ -1931,8 +1931,13 @@ cudaError_t launch_rows(const SweepArgs& a, cudaStream_t s) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
-  if (smem + ROWS_STAGES * sizeof(uint64_t) > size_t(optin)) return cudaErrorNotSupported;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  // the ring of the longest rows that fit beside the barriers (nx % 8 == 0). The limit belongs
+  // to the kernel, not to the launch, and other threads may be launching it for rows of
+  // another length, so it is always this one.
+  const size_t step = size_t(ROWS_STAGES) * Q * 8 * sizeof(__half);
+  const size_t most = (size_t(optin) - 2 * ROWS_STAGES * sizeof(uint64_t)) / step * step;
+  if (smem > most) return cudaErrorNotSupported;
+  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(most));
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, ROWS_THREADS, smem);
   if (e != cudaSuccess) return e;
   if (per < 1) return cudaErrorNotSupported;

@@ -207,7 +207,10 @@ cudaError_t launch_resident_geom(const SweepArgs& a, int steps, bool swapped, cu
   const uint32_t more = std::is_same<S, double>::value ? (per + 127u) / 128u * 128u : per + 256u;
   const uint32_t threads = more < RESIDENT_THREADS ? more : RESIDENT_THREADS;
   const size_t smem = size_t(2) * Q * per * sizeof(S);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  // The limit belongs to the kernel, not to the launch, and other threads may be launching it
+  // for lattices of other sizes: always the largest lattice's (77,824 bytes; binary16 half).
+  constexpr uint32_t most = (std::is_same<S, double>::value ? RESIDENT_NODES_F64 : RESIDENT_NODES) / RESIDENT_CTAS;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(2 * Q * most * sizeof(S)));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
