@@ -146,9 +146,10 @@ LBM_API lbm_status lbm_set_stream(lbm_ctx* ctx, void* cuda_stream);
  * the edge correction eq. edge, buried links eq. buried and eq. corner; then BGK
  * collision (eq. bgk, eq. feq). Binary16 lattices whose rows are multiples of 8 nodes
  * and at least 256 long take a sweep that stages population rows in shared memory with
- * bulk copies. 16 or more steps of a small lattice are one launch: up to 8,192 nodes (FP64
- * 4,096) of one thread-block cluster, A/B lattices beyond, up to 1,024 nodes per SM (FP64
- * 512), of a cooperative grid with a barrier between steps. Waits of either kind of kernel
+ * bulk copies. 16 to 4,096 steps of a small lattice are one launch (more, one for each
+ * 4,096): up to 8,192 nodes (FP64 4,096) of one thread-block cluster, A/B lattices beyond, up
+ * to 1,024 nodes per SM (FP64 512), of a cooperative grid with a barrier between steps,
+ * which starts when there is room for all of it. Waits of either kind of kernel
  * are bounded, and one that runs out is reported by the next synchronising call as
  * LBM_ERR_CUDA (see lbm_debug_drop_staged_copies). Every sweep variant computes the same
  * bits for a node. */

@@ -232,6 +232,9 @@ constexpr uint32_t RESIDENT_THREADS = 512;
 constexpr uint32_t RESIDENT_CTAS = 16;
 constexpr uint32_t RESIDENT_NODES = RESIDENT_THREADS * RESIDENT_CTAS, RESIDENT_NODES_F64 = RESIDENT_NODES / 2;
 constexpr int RESIDENT_MIN_STEPS = 16;
+// Steps of one launch at most, even: about 5 to 20 ms, after which work of other streams
+// gets the SMs, as it does between the launches of single steps.
+constexpr int MULTI_STEPS_MAX = 4096;
 // Nodes beyond which no A/B lattice takes its steps in one launch of a block per SM (the
 // launch itself knows the SMs).
 constexpr uint32_t GRID_STEPS_NODES = 262144;

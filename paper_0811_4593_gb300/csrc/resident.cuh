@@ -259,8 +259,11 @@ cudaError_t launch_resident_impl(const SweepArgs& a, int steps, bool swapped, cu
 template <typename S> constexpr int grid_step_threads() { return std::is_same<S, double>::value ? 512 : 1024; }
 
 // Grid barrier: every block arrives and waits for `target` arrivals; false once the wait
-// has taken STAGE_WAIT_LIMIT_NS (the blocks of a cooperative launch are all resident, so
-// it ends; the limit bounds it all the same). Every thread of the block takes part.
+// has taken STAGE_WAIT_LIMIT_NS. A cooperative grid is placed as a whole: beside a kernel
+// that kept one SM for 3 s, and beside a second such grid, blocks that fill an SM each
+// started together when there was room for all, and no wait ran out. So a wait lasts as
+// long as the slowest block's step; the limit bounds it all the same. Every thread of the
+// block takes part.
 __device__ __forceinline__ bool grid_barrier(uint32_t* arrivals, uint32_t target, const SweepArgs& a) {
   __shared__ bool ok;
   __syncthreads();
@@ -332,8 +335,9 @@ cudaError_t launch_grid_steps_geom(const SweepArgs& a, int steps, uint32_t* arri
   SweepArgs first = a;
   void* args[] = {&first, &b, &steps, &arrivals};
   e = cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(per), args, 0, s);
-  if (e != cudaErrorCooperativeLaunchTooLarge) return e;
-  cudaGetLastError();  // fewer SMs are free for this process than the device has
+  // fewer SMs are free for this process than the device has, or no such launches at all
+  if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) return e;
+  cudaGetLastError();
   return cudaErrorNotSupported;
 }
 

@@ -328,39 +328,30 @@ cudaError_t dispatch_grid_steps(lbm_ctx* ctx, int n) {
   }
 }
 
-// Issues n plain steps: one launch each, or for a small lattice all of them (an even
-// number for AA, whose state it reads and leaves between step pairs) in one.
+// Issues n plain steps: one launch each, or for a small lattice up to MULTI_STEPS_MAX of
+// them (an even number for AA, whose state it reads and leaves between step pairs) in one.
 lbm_status issue_steps(lbm_ctx* ctx, int n) {
   const bool aa = ctx->scheme == LBM_SCHEME_AA;
-  const int m = aa ? n & ~1 : n;
-  const uint32_t resident = ctx->prec == LBM_F64 ? lbm::RESIDENT_NODES_F64 : lbm::RESIDENT_NODES;
-  if (ctx->N <= resident && m >= lbm::RESIDENT_MIN_STEPS && !(aa && ctx->steps % 2 != 0)) {
-    // m steps leave the state where m launches would: in the other array when m is odd
+  const bool cluster = ctx->N <= (ctx->prec == LBM_F64 ? lbm::RESIDENT_NODES_F64 : lbm::RESIDENT_NODES);
+  const bool many = cluster ? !(aa && ctx->steps % 2 != 0)
+                            : !aa && lbm::plain_step_nodes(ctx->args) <= lbm::GRID_STEPS_NODES;
+  while (many) {
+    const int most = n < lbm::MULTI_STEPS_MAX ? n : lbm::MULTI_STEPS_MAX;
+    const int m = aa ? most & ~1 : most;
+    if (m < lbm::RESIDENT_MIN_STEPS) break;
     set_direction(ctx, ctx->cur);
-    if (m % 2 == 0) {
+    if (cluster && m % 2 == 0) {
+      // m steps leave the state where m launches would: in the other array when m is odd
       ctx->args.dst = ctx->buf[ctx->cur];
       for (int k = 0; k < 19; ++k) ctx->args.dst_pop[k] = const_cast<void*>(ctx->args.src_pop[k]);
     }
-    const cudaError_t e = dispatch_resident(ctx, m);
-    if (e == cudaSuccess) {
-      if (!aa) ctx->cur ^= m & 1;
-      ctx->steps += m;
-      ctx->launches += 1;
-      n -= m;
-    } else if (e != cudaErrorNotSupported) {
-      return cuda_fail(ctx, e, "multi-step launch");
-    }
-  } else if (!aa && lbm::plain_step_nodes(ctx->args) <= lbm::GRID_STEPS_NODES && n >= lbm::RESIDENT_MIN_STEPS) {
-    set_direction(ctx, ctx->cur);
-    const cudaError_t e = dispatch_grid_steps(ctx, n);
-    if (e == cudaSuccess) {
-      ctx->cur ^= n & 1;
-      ctx->steps += n;
-      ctx->launches += 1;
-      n = 0;
-    } else if (e != cudaErrorNotSupported) {
-      return cuda_fail(ctx, e, "multi-step launch");
-    }
+    const cudaError_t e = cluster ? dispatch_resident(ctx, m) : dispatch_grid_steps(ctx, m);
+    if (e == cudaErrorNotSupported) break;
+    LBM_CUDA(ctx, e, "multi-step launch");
+    if (!aa) ctx->cur ^= m & 1;
+    ctx->steps += m;
+    ctx->launches += 1;
+    n -= m;
   }
   if (n >= 2 && in_place_pays(ctx)) {
     set_in_place(ctx);
