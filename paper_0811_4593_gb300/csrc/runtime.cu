@@ -8,6 +8,7 @@
 #include <cstddef>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
@@ -51,8 +52,9 @@ struct lbm_ctx {
   double* dred = nullptr;    // reduction results [4], and behind them
   uint32_t* derr = nullptr;  // the error word of the sweeps (SweepArgs::err)
   uint32_t* dticket = nullptr;  // and the fold's ticket
-  uint2* fluid = nullptr;       // list of fluid nodes, N entries allocated (SweepArgs::fluid)
   uint32_t* darrivals = nullptr;  // and the arrivals of the multi-step kernel's grid barrier
+  uint32_t* links = nullptr;      // geometry words, N allocated (SweepArgs::links)
+  uint2* fluid = nullptr;         // list of fluid nodes, N entries allocated (SweepArgs::fluid)
   cudaStream_t stream = nullptr;
   int64_t steps = 0, launches = 0, device_bytes = 0;
   int64_t l2_bytes = 0;
@@ -810,29 +812,30 @@ lbm_status lbm_set_geometry(lbm_ctx* ctx, const uint8_t* solid, const int8_t* co
         // overwritten (a solid source may hold anything)
         links[node] = (rule << lbm::RULE_SHIFT) | rule_mask;
       }
-  if (!ctx->args.links) {
-    void* d = ctx_alloc(ctx, sizeof(uint32_t) * ctx->N);
-    if (!d) return fail(ctx, LBM_ERR_OOM, "allocation of the geometry words failed");
-    ctx->args.links = static_cast<const uint32_t*>(d);
-  }
-  LBM_CUDA(ctx, cudaMemcpyAsync(const_cast<uint32_t*>(ctx->args.links), links.data(), sizeof(uint32_t) * ctx->N,
-                                cudaMemcpyHostToDevice, ctx->stream), "uploading the geometry words");
+  if (!ctx->links) ctx->links = static_cast<uint32_t*>(ctx_alloc(ctx, sizeof(uint32_t) * ctx->N));
+  if (!ctx->links) return fail(ctx, LBM_ERR_OOM, "allocation of the geometry words failed");
   // Fluid nodes as a list where at least an eighth of the nodes are solid: its 8 bytes a
   // node in place of 4 are paid back by the solid nodes' idle lanes (128 x 16 x 256, two
-  // thirds solid, FP32: 10.5 us a step without, 7.3 with).
-  std::vector<uint2> fluid;
-  for (uint32_t i = 0; i < ctx->N; ++i)
-    if (!(links[i] & lbm::SOLID_NODE)) fluid.push_back(make_uint2(i, links[i]));
-  const bool list = fluid.size() <= ctx->N - ctx->N / 8;
-  if (list && !ctx->fluid) {
-    ctx->fluid = static_cast<uint2*>(ctx_alloc(ctx, sizeof(uint2) * ctx->N));
-    if (!ctx->fluid) return fail(ctx, LBM_ERR_OOM, "allocation of the list of fluid nodes failed");
-  }
+  // thirds solid, FP32: 10.5 us a step without, 7.3 with). Without the memory for it the
+  // steps do without.
+  uint32_t nfluid = 0;
+  for (uint32_t word : links) nfluid += (word & lbm::SOLID_NODE) ? 0u : 1u;
+  bool list = nfluid <= ctx->N - ctx->N / 8;
+  if (list && !ctx->fluid) ctx->fluid = static_cast<uint2*>(ctx_alloc(ctx, sizeof(uint2) * ctx->N));
+  std::unique_ptr<uint2[]> fluid(list && ctx->fluid ? new (std::nothrow) uint2[nfluid] : nullptr);
+  list = fluid != nullptr;
+  if (list)
+    for (uint32_t i = 0, n = 0; i < ctx->N; ++i)
+      if (!(links[i] & lbm::SOLID_NODE)) fluid[n++] = make_uint2(i, links[i]);
+  // nothing fails for want of memory from here on: the geometry is in force as a whole
+  LBM_CUDA(ctx, cudaMemcpyAsync(ctx->links, links.data(), sizeof(uint32_t) * ctx->N, cudaMemcpyHostToDevice, ctx->stream),
+           "uploading the geometry words");
+  if (nfluid && list)
+    LBM_CUDA(ctx, cudaMemcpyAsync(ctx->fluid, fluid.get(), sizeof(uint2) * nfluid, cudaMemcpyHostToDevice, ctx->stream),
+             "uploading the list of fluid nodes");
+  ctx->args.links = ctx->links;
   ctx->args.fluid = list ? ctx->fluid : nullptr;
-  ctx->args.nfluid = list ? uint32_t(fluid.size()) : 0u;
-  if (list && !fluid.empty())
-    LBM_CUDA(ctx, cudaMemcpyAsync(ctx->fluid, fluid.data(), sizeof(uint2) * fluid.size(), cudaMemcpyHostToDevice,
-                                  ctx->stream), "uploading the list of fluid nodes");
+  ctx->args.nfluid = list ? nfluid : 0u;
   // solid nodes keep their populations, and plain steps leave them alone in both arrays:
   // start both alike
   LBM_CUDA(ctx, cudaMemcpyAsync(ctx->buf[ctx->cur ^ 1], ctx->buf[ctx->cur], 19ull * ctx->N * storage_bytes(ctx->prec),
