@@ -190,6 +190,8 @@ LBM_API lbm_status lbm_get_populations(lbm_ctx* ctx, void* dst, int z0, int nzs,
  * Solid nodes keep their populations; plain steps neither read nor write them. Costs 4
  * bytes per node of extra traffic per step, or where an eighth or more of the nodes are
  * solid 8 bytes per fluid node (a list of them, 8 bytes per node of device memory).
+ * Steps captured in a CUDA graph while a geometry is set read the words only, and replay
+ * with the geometry last set.
  * A/B scheme only (LBM_ERR_ARG for AA). Synchronises. */
 LBM_API lbm_status lbm_set_solid(lbm_ctx* ctx, const uint8_t* solid);
 

@@ -55,6 +55,7 @@ struct lbm_ctx {
   uint32_t* darrivals = nullptr;  // and the arrivals of the multi-step kernel's grid barrier
   uint32_t* links = nullptr;      // geometry words, N allocated (SweepArgs::links)
   uint2* fluid = nullptr;         // list of fluid nodes, N entries allocated (SweepArgs::fluid)
+  bool fluid_list = false;        // the geometry in force has its list there
   cudaStream_t stream = nullptr;
   int64_t steps = 0, launches = 0, device_bytes = 0;
   int64_t l2_bytes = 0;
@@ -330,9 +331,21 @@ cudaError_t dispatch_grid_steps(lbm_ctx* ctx, int n) {
   }
 }
 
+// Has plain steps visit the fluid nodes by their list, if there is one, unless they are
+// being captured: a captured launch keeps the list's length, while the next lbm_set_geometry
+// rewrites the list and the words in place. By the words alone (128 x 16 x 256, two thirds
+// solid, FP32: 10.5 us a step, with the list 7.3) a replay has the geometry then in force.
+lbm_status choose_nodes(lbm_ctx* ctx) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (ctx->fluid_list) LBM_CUDA(ctx, cudaStreamIsCapturing(ctx->stream, &capture), "asking whether the stream captures");
+  ctx->args.fluid = ctx->fluid_list && capture == cudaStreamCaptureStatusNone ? ctx->fluid : nullptr;
+  return LBM_OK;
+}
+
 // Issues n plain steps: one launch each, or for a small lattice up to MULTI_STEPS_MAX of
 // them (an even number for AA, whose state it reads and leaves between step pairs) in one.
 lbm_status issue_steps(lbm_ctx* ctx, int n) {
+  if (lbm_status st = choose_nodes(ctx); st != LBM_OK) return st;
   const bool aa = ctx->scheme == LBM_SCHEME_AA;
   const bool cluster = ctx->N <= (ctx->prec == LBM_F64 ? lbm::RESIDENT_NODES_F64 : lbm::RESIDENT_NODES);
   const bool many = cluster ? !(aa && ctx->steps % 2 != 0)
@@ -834,7 +847,7 @@ lbm_status lbm_set_geometry(lbm_ctx* ctx, const uint8_t* solid, const int8_t* co
     LBM_CUDA(ctx, cudaMemcpyAsync(ctx->fluid, fluid.get(), sizeof(uint2) * nfluid, cudaMemcpyHostToDevice, ctx->stream),
              "uploading the list of fluid nodes");
   ctx->args.links = ctx->links;
-  ctx->args.fluid = list ? ctx->fluid : nullptr;
+  ctx->fluid_list = list;
   ctx->args.nfluid = list ? nfluid : 0u;
   // solid nodes keep their populations, and plain steps leave them alone in both arrays:
   // start both alike
