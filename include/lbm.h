@@ -50,9 +50,14 @@ typedef enum {
 } lbm_status;
 
 /* Storage of the populations and the arithmetic of the sweep.
- *  LBM_F64          f_i stored as double; arithmetic in 64-bit fixed point, at least as
- *                   exact as in double, on nodes whose populations lie near a flow's
- *                   (see fixed64.cuh), in double on any other; reductions in double.
+ *  LBM_F64          f_i stored as double; arithmetic in 64-bit fixed point on nodes whose
+ *                   populations lie near a flow's (see fixed64.cuh), in double on any
+ *                   other; reductions in double. The error of fixed point is absolute,
+ *                   about half the last place of the rest population: for tau <= 3 it is
+ *                   by rms no larger than double's for any population; at longer
+ *                   relaxation times populations below rho0 / 32 (for rho0 a power of two
+ *                   rho0 / 64) may have up to three bits less than in double, the others
+ *                   and the node's sums have more.
  *  LBM_F32          shifted populations h_i = f_i - w_i rho0 stored as float;
  *                   arithmetic in float except the density of a face closure (eq. uin
  *                   and its appendix analogues), which is formed as a float pair,
