@@ -41,7 +41,7 @@ __device__ __forceinline__ bool fixed_close_face(int64_t (&f)[Q], const FixedFac
   });
   const int64_t s = in + (out + out);
   const int64_t d = pressure ? v.r - s : mul63(s, limbs_of(v.r)) * 2;
-  const int64_t rho = s + d;
+  const int64_t rho = int64_t(uint64_t(s) + uint64_t(d));  // below 2^64: negative where it does not fit
   const int64_t third = mul63(d, limbs_of(fixed_part(3)));
   auto tangent = [&](auto tc, int64_t factor) {
     constexpr int T = decltype(tc)::value;
