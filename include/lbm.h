@@ -61,7 +61,8 @@ typedef enum {
  *  LBM_F32          shifted populations h_i = f_i - w_i rho0 stored as float;
  *                   arithmetic in float except the density of a face closure (eq. uin
  *                   and its appendix analogues), which is formed as a float pair,
- *                   and the reductions, which accumulate as float pairs and in double.
+ *                   and the reductions, which accumulate as sums of three floats (as
+ *                   exact as in double) and in double.
  *  LBM_F16_SHIFTED  h_i = f_i - w_i rho0 stored as IEEE binary16 (round to nearest
  *                   even); arithmetic as for LBM_F32. */
 typedef enum { LBM_F64 = 0, LBM_F32 = 1, LBM_F16_SHIFTED = 2 } lbm_precision;
@@ -160,7 +161,7 @@ LBM_API lbm_status lbm_set_stream(lbm_ctx* ctx, void* cuda_stream);
  * bits for a node. */
 LBM_API lbm_status lbm_step(lbm_ctx* ctx, int n);
 
-/* Advance n >= 1 steps like lbm_step, the last one also forming, in double, the
+/* Advance n >= 1 steps like lbm_step, the last one also forming, to double precision, the
  * total mass sum(rho) and the steady-state residual
  *   r = sqrt(sum |u - u_snap|^2) / sqrt(sum |u|^2)
  * where u_snap is the velocity field at the previous residual evaluation (zero

@@ -928,29 +928,61 @@ __device__ __forceinline__ double warp_terms_f64(const NodeTerms<T>& t, bool act
   return warp_sum4(q[0], q[1], q[2], q[3]);
 }
 
-// hi + lo of (a - b)^2 for a difference taken exactly (TwoSum), to about 2^-47
-__device__ __forceinline__ fpair square_diff(float a, float b) {
-  const float d = __fsub_rn(a, b);
-  const float bb = __fsub_rn(d, a);
-  const float e = __fsub_rn(__fsub_rn(a, __fsub_rn(d, bb)), __fadd_rn(b, bb));
-  const float h = __fmul_rn(d, d);
-  return {h, __fmaf_rn(__fmul_rn(2.0f, d), e, __fmaf_rn(d, d, -h))};
+// (a - b)^2 for a difference taken exactly, d + e: d^2 + 2 d e + e^2, to about 2^-72
+__device__ __forceinline__ ftriple square_diff(float a, float b) {
+  const fpair d = two_sum(a, -b);
+  const float h = __fmul_rn(d.hi, d.hi), twice = __fmul_rn(2.0f, d.hi);
+  const float m = __fmul_rn(twice, d.lo);
+  const fpair l = two_sum(__fmaf_rn(d.hi, d.hi, -h), m);
+  return {h, l.hi, __fadd_rn(l.lo, __fmaf_rn(d.lo, d.lo, __fmaf_rn(twice, d.lo, -m)))};
 }
-__device__ __forceinline__ fpair square(float a) {
+__device__ __forceinline__ ftriple square(float a) {
   const float h = __fmul_rn(a, a);
-  return {h, __fmaf_rn(a, a, -h)};
+  return {h, __fmaf_rn(a, a, -h), 0.0f};
+}
+
+// Two triples as one operand of the packed instructions (additions only: every lane rounds as
+// the scalar sum_of does).
+struct ftriple2 {
+  f32x2 hi, lo, rest;
+  __device__ ftriple2(ftriple a, ftriple b) : hi(a.hi, b.hi), lo(a.lo, b.lo), rest(a.rest, b.rest) {}
+  __device__ ftriple2(f32x2 h, f32x2 l, f32x2 r) : hi(h), lo(l), rest(r) {}
+  __device__ ftriple first() const { return {hi.x, lo.x, rest.x}; }
+  __device__ ftriple second() const { return {hi.y, lo.y, rest.y}; }
+};
+__device__ __forceinline__ ftriple2 sum_of(ftriple2 a, ftriple2 b) {
+  auto error = [](f32x2 x, f32x2 y, f32x2 s) {  // of s = x + y (TwoSum)
+    const f32x2 t = op_sub(s, x);
+    return op_add(op_sub(x, op_sub(s, t)), op_sub(y, t));
+  };
+  const f32x2 s = op_add(a.hi, b.hi), e = error(a.hi, b.hi, s);
+  const f32x2 t = op_add(a.lo, b.lo), f = error(a.lo, b.lo, t);
+  const f32x2 l = op_add(t, e), g = error(t, e, l);
+  return {s, l, op_add(op_add(a.rest, b.rest), op_add(f, g))};
+}
+// warp_sum4 with its first step in packed pairs.
+__device__ __forceinline__ ftriple warp_sum4(ftriple2 q01, ftriple2 q23) {
+  const bool up = threadIdx.x & 16, up2 = threadIdx.x & 8;
+  const ftriple2 own = up ? q23 : q01, other = up ? q01 : q23;
+  const ftriple2 k = sum_of(own, ftriple2(shfl_xor(other.first(), 16), shfl_xor(other.second(), 16)));
+  ftriple s = sum_of(up2 ? k.second() : k.first(), shfl_xor(up2 ? k.first() : k.second(), 8));
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) s = sum_of(s, shfl_xor(s, o));
+  return s;
 }
 
 // Block sums of the residual reductions over the active threads of block `blk` (nodes
 // blk*256 .. of N), into out[4]; every thread of the block takes part. The snapshot takes
-// the velocities. Float lattices form the node terms and
-// the warp sums as float pairs (about 48 bits): in double they were 45 FP64 instructions
-// per warp, about 850 SM cycles against 260 for the memory traffic of its nodes. The
-// velocities are scaled by 2^32 so that squares neither overflow nor lose their low
-// parts; a warp with a value outside the range that this covers (|u| >= 2^26, a density
-// deviation beyond 2^64, not-a-number, or a largest velocity or change below 2^-72 that
-// is not zero) forms its sums in double. So do FP64 lattices. The warp results are
-// added in double in either case.
+// the velocities. Float lattices form the node terms and the warp sums as unevaluated sums
+// of three floats (exact to about 2^-70, so the results are as exact as sums in double): in
+// double they were 45 FP64 instructions per warp, about 850 SM cycles against 260 for the
+// memory traffic of its nodes. (512 x 512 x 256: a residual step 2.04 ms in FP32, 1.91 in
+// binary16; with two floats, whose sums were 4 to 20 units of 2^-53 off, 1.91 and 1.71.) The
+// velocities are scaled by 2^32 so that squares neither overflow nor lose their low parts; a
+// warp with a value outside the range that this covers (|u| >= 2^26, a density deviation
+// beyond 2^64, not-a-number, or a largest velocity or change below 2^-72 that is not zero)
+// forms its sums in double. So do FP64 lattices. The warp results are added in double in
+// either case.
 template <typename T>
 __device__ __forceinline__ void block_terms(const NodeTerms<T>& t, uint32_t N, uint32_t blk, double rho0,
                                             float neg_rho0, T* snap, double* out) {
@@ -971,8 +1003,8 @@ __device__ __forceinline__ void block_terms(const NodeTerms<T>& t, uint32_t N, u
       if (lane < 4) out[lane] = v;
     }
   } else {
-    __shared__ fpair pairs[WARPS][4];
-    __shared__ bool in_pairs[WARPS];
+    __shared__ ftriple parts[WARPS][4];
+    __shared__ bool in_parts[WARPS];
     float u[3], p[3], drho = 0.0f;
     bool ok = true, range = true;
     float big = 0.0f, step = 0.0f;
@@ -998,23 +1030,25 @@ __device__ __forceinline__ void block_terms(const NodeTerms<T>& t, uint32_t N, u
     const uint32_t least = __float_as_uint(0x1p-40f);
     if (__all_sync(0xffffffffu, range) && (bits_u == 0u || bits_u >= least) && (bits_d == 0u || bits_d >= least)) {
       const uint32_t bad = __popc(__ballot_sync(0xffffffffu, !ok));
-      const fpair d2 = sum_of(sum_of(square_diff(u[0], p[0]), square_diff(u[1], p[1])), square_diff(u[2], p[2]));
-      const fpair u2 = sum_of(sum_of(square(u[0]), square(u[1])), square(u[2]));
-      const fpair k = warp_sum4(fpair{drho, 0.0f}, d2, u2, fpair{0.0f, 0.0f});
-      if ((lane & 7) == 0) pairs[warp][lane >> 3] = lane == 24 ? fpair{float(bad), 0.0f} : k;
-      if (lane == 0) in_pairs[warp] = true;
+      auto squares = [&](int i) { return ftriple2(square_diff(u[i], p[i]), square(u[i])); };
+      const ftriple2 q = sum_of(sum_of(squares(0), squares(1)), squares(2));  // |u - p|^2, |u|^2
+      const ftriple none = {0.0f, 0.0f, 0.0f};
+      const ftriple k = warp_sum4(ftriple2(ftriple{drho, 0.0f, 0.0f}, q.first()), ftriple2(q.second(), none));
+      if ((lane & 7) == 0) parts[warp][lane >> 3] = lane == 24 ? ftriple{float(bad), 0.0f, 0.0f} : k;
+      if (lane == 0) in_parts[warp] = true;
     } else {
       const double k = warp_terms_f64(t, active, rho0);
       if ((lane & 7) == 0) sums[warp][lane >> 3] = k;
-      if (lane == 0) in_pairs[warp] = false;
+      if (lane == 0) in_parts[warp] = false;
     }
     __syncthreads();
     if (active) store_snapshot(t, snap, N, cell);
     if (warp == 0) {
       const int w = lane >> 2, j = lane & 3;
       double v;
-      if (in_pairs[w]) {
-        v = double(pairs[w][j].hi) + double(pairs[w][j].lo);
+      if (in_parts[w]) {
+        const ftriple p = parts[w][j];
+        v = double(p.hi) + (double(p.lo) + double(p.rest));
         if (j == 1 || j == 2) v = op_mul(v, 0x1p-64);
       } else {
         v = sums[w][j];
@@ -1293,9 +1327,9 @@ __device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk, ui
 template <typename S, bool RESID, bool BATCHED, int MODE, bool GEOM = false>
 struct SweepOccupancy {
   static constexpr int base = RESID ? 5 : 6;
-  static constexpr int aa = std::is_same<S, float>::value && !BATCHED ? 4 + MODE
-                            : MODE == 1                               ? 4
-                                                                      : 5;
+  static constexpr int aa = std::is_same<S, float>::value && !BATCHED && !RESID ? 4 + MODE
+                            : MODE == 1                                         ? 4
+                                                                                : 5;
   static constexpr int blocks = GEOM ? 4 : (MODE == 0 ? base : aa);
 };
 template <bool RESID, bool BATCHED, int MODE, bool GEOM>
