@@ -228,9 +228,15 @@ __host__ __device__ __forceinline__ void fixed_relax_to(const int64_t (&f)[19], 
   }
 }
 
+// UNIT: ask whether omega is 1. A kernel then holds two bodies, which is free in the plain
+// single-lattice A/B steps (256 x 64 x 64 at tau = 0.6 65.0 us with and without, at tau = 1
+// 56.9 against 65.0), but not in those that spill or hold more beside it: AA steps at other
+// tau 1,109 against 1,101 us (256^3), batches 466 against 453 us a step (ten lattices of 40
+// to 150 nodes a side); they go without.
+template <bool UNIT = true>
 __host__ __device__ __forceinline__ void fixed_relax(const int64_t (&f)[19], const FixedSums& q, const FixedArgs& fx,
                                                      double (&h)[19]) {
-  if ((fx.keep[0] | fx.keep[1]) == 0) fixed_relax_to<false>(f, q, fx, h);
+  if (UNIT && (fx.keep[0] | fx.keep[1]) == 0) fixed_relax_to<false>(f, q, fx, h);
   else fixed_relax_to<true>(f, q, fx, h);
 }
 

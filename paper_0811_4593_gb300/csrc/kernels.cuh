@@ -1150,7 +1150,7 @@ __device__ __forceinline__ void relax_node(const SweepArgs& a, T (&h)[Q], uint32
 
 // Closure and relaxation of an FP64 node in fixed point; false, with h in no particular
 // state, where the node has to be taken in double.
-template <bool RESID, bool GEOM>
+template <bool RESID, bool GEOM, bool UNIT>
 __device__ __forceinline__ bool update_fixed(const SweepArgs& a, uint32_t lm, int code, uint32_t x, uint32_t y, uint32_t z,
                                              uint32_t cell, double (&h)[Q], NodeTerms<double>& terms) {
   if (GEOM && (lm & SOLID_NODE)) return false;
@@ -1169,20 +1169,20 @@ __device__ __forceinline__ bool update_fixed(const SweepArgs& a, uint32_t lm, in
       q.z += a.fx.force[2];
     }
   }
-  fixed_relax(f, q, a.fx, h);
+  fixed_relax<UNIT>(f, q, a.fx, h);
   return true;
 }
 
 // One node: load(h) fetches its streamed populations, on return h holds the new ones. FP64
 // nodes go through fixed point where they can; the few others are loaded again, which
-// keeps their doubles from occupying registers meanwhile.
-template <typename S, bool RESID, bool GEOM, typename T, typename Load>
+// keeps their doubles from occupying registers meanwhile. UNIT: see fixed_relax.
+template <typename S, bool RESID, bool GEOM, bool UNIT, typename T, typename Load>
 __device__ __forceinline__ void update_node(const SweepArgs& a, uint32_t lm, int code, uint32_t x, uint32_t y, uint32_t z,
                                             uint32_t cell, Load&& load, T (&h)[Q], NodeTerms<T>& terms) {
   load(h);
   if constexpr (std::is_same<T, double>::value) {
     if (a.fx.on) {
-      if (update_fixed<RESID, GEOM>(a, lm, code, x, y, z, cell, h, terms)) return;
+      if (update_fixed<RESID, GEOM, UNIT>(a, lm, code, x, y, z, cell, h, terms)) return;
       load(h);
     }
   }
@@ -1222,7 +1222,7 @@ enum StreamMode : int { STREAM_AB = 0, STREAM_AA_GATHER = 1, STREAM_AA_LOCAL = 2
 // lbm_set_populations), so a plain step neither reads nor writes it.
 // COHERENT: the source array is written by other blocks of the same launch (between grid
 // barriers), so it is read through L2.
-template <typename S, bool RESID, int MODE, bool GEOM = false, bool COHERENT = false, typename T>
+template <typename S, bool RESID, int MODE, bool GEOM = false, bool COHERENT = false, bool UNIT = false, typename T>
 __device__ __forceinline__ void sweep_node(const SweepArgs& a, uint32_t cell, uint32_t lm, NodeTerms<T>& terms) {
   if (cell < a.N && (!GEOM || RESID || !(lm & SOLID_NODE))) {
     const uint32_t q1 = fdiv(a.div_nx, cell);
@@ -1280,7 +1280,7 @@ __device__ __forceinline__ void sweep_node(const SweepArgs& a, uint32_t cell, ui
     const int fz = pz ? 0 : (z == 0 ? 1 : (z == a.nz - 1 ? 2 : 0));
     const int code = fx + 3 * fy + 9 * fz;
     T h[Q];
-    update_node<S, RESID, GEOM>(a, lm, code, x, y, z, cell, load, h, terms);
+    update_node<S, RESID, GEOM, UNIT>(a, lm, code, x, y, z, cell, load, h, terms);
     static_for<0, Q>([&](auto kc) {
       constexpr int k = decltype(kc)::value;
       if constexpr (MODE == STREAM_AB) {
@@ -1301,11 +1301,11 @@ __device__ __forceinline__ void sweep_node(const SweepArgs& a, uint32_t cell, ui
 }
 
 // Block `blk` (nodes blk*256 .. blk*256+255).
-template <typename S, bool RESID, int MODE, bool GEOM = false>
+template <typename S, bool RESID, int MODE, bool GEOM = false, bool UNIT = false>
 __device__ __forceinline__ void sweep_block(const SweepArgs& a, uint32_t blk, uint32_t lm = 0u) {
   using T = typename ComputeOf<S>::T;
   NodeTerms<T> terms = {};
-  sweep_node<S, RESID, MODE, GEOM>(a, blk * SWEEP_THREADS + threadIdx.x, lm, terms);
+  sweep_node<S, RESID, MODE, GEOM, false, UNIT>(a, blk * SWEEP_THREADS + threadIdx.x, lm, terms);
   if constexpr (RESID)
     block_terms(terms, a.N, blk, ref_rho<S>(a.rho0), a.neg_rho0, static_cast<T*>(a.snap), a.partials + 4ull * blk);
 }
@@ -1347,14 +1347,14 @@ __global__ void __launch_bounds__(SWEEP_THREADS, (SweepOccupancy<S, RESID, false
     uint2 node = geometry_node(a, blk * SWEEP_THREADS + threadIdx.x);
     wait_for_previous_sweep(node.x, node.y);
     NodeTerms<typename ComputeOf<S>::T> unused;
-    sweep_node<S, false, MODE, true>(a, node.x, node.y, unused);
+    sweep_node<S, false, MODE, true, false, true>(a, node.x, node.y, unused);
   } else if constexpr (GEOM) {
     uint32_t lm = geometry_word(a, blk * SWEEP_THREADS + threadIdx.x);
     wait_for_previous_sweep(blk, lm);
     sweep_block<S, RESID, MODE, GEOM>(a, blk, lm);
   } else {
     wait_for_previous_sweep(blk);
-    sweep_block<S, RESID, MODE, GEOM>(a, blk);
+    sweep_block<S, RESID, MODE, GEOM, MODE == STREAM_AB && !RESID>(a, blk);
   }
 }
 

@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(RESIDENT_THREADS, 1)
         static_for<0, Q>([&](auto kc) { v[decltype(kc)::value] = ld_cluster(from[decltype(kc)::value] + array, S()); });
       };
       NodeTerms<T> unused;
-      update_node<S, false, GEOM>(a, lm, code, x, y, z, cell, load, h, unused);
+      update_node<S, false, GEOM, true>(a, lm, code, x, y, z, cell, load, h, unused);
       if (last) {
         static_for<0, Q>([&](auto kc) {
           constexpr int k = decltype(kc)::value;
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__((grid_step_threads<S>()), 1)
   }
   NodeTerms<typename ComputeOf<S>::T> unused;
   for (int s = 0;;) {
-    sweep_node<S, false, STREAM_AB, GEOM, true>((s & 1) ? b : a, cell, lm, unused);
+    sweep_node<S, false, STREAM_AB, GEOM, true, true>((s & 1) ? b : a, cell, lm, unused);
     if (++s == steps) break;
     if (!grid_barrier(arrivals, uint32_t(s) * gridDim.x, a)) break;
   }
