@@ -26,13 +26,15 @@ COMPUTE_BYTES = {"f64": 8, "f32": 4, "f16": 4}
 
 def footprint_bytes(nx: int, ny: int, nz: int, precision: str, scheme: str = "ab") -> int:
     """Device bytes one resident lattice holds: its population buffers (two for the A/B
-    scheme, one for AA), the residual snapshot and partial sums, the face tables and the
-    reduction scalars."""
+    scheme, one for AA), the residual snapshot and partial sums (a row of four doubles for
+    each 256 nodes and, of their fold, for each 1,024 such rows), tables on all faces, and
+    the reduction results with the sweeps' words."""
     n = nx * ny * nz
     blocks = (n + 255) // 256
+    rows = blocks + (blocks + 1023) // 1024
     faces = 2 * (ny * nz + nx * nz + nx * ny) * 64
     buffers = 1 if scheme == "aa" else 2
-    return buffers * 19 * STORAGE_BYTES[precision] * n + 3 * COMPUTE_BYTES[precision] * n + 32 * blocks + faces + 32
+    return buffers * 19 * STORAGE_BYTES[precision] * n + 3 * COMPUTE_BYTES[precision] * n + 32 * rows + faces + 44
 
 
 @dataclass
