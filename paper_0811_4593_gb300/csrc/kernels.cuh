@@ -262,7 +262,10 @@ __device__ __forceinline__ void two_sum_acc(f32x2& hi, f32x2& lo, f32x2 t) {
 // in float ones. The FP64 pipe issues a warp instruction in about 19 SM cycles, so the
 // six conversions and operations that formed a float node's density in double took half
 // of a face node's time in short-row and small lattices; rounded to float, the pair's
-// result differs from the double one in about one of 2^21 cases, by one ulp.
+// result differs from the double one in about one of 2^21 cases, by one ulp. The normal
+// velocity of a pressure plane, rms against the exact one in units of the populations, pair
+// and double: 8.0e-8 both for populations of 1e-2 to 1e-6, 1.1e-7 and 0.8e-7 for 1e-8 (the
+// last place of 1, against which it cancels), 1.0e-6 and 1.1e-6 for 6e-11.
 template <typename T> struct WideOf { using type = double; };
 template <> struct WideOf<float> { using type = fpair; };
 template <typename T> using Wide = typename WideOf<T>::type;
